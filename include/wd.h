@@ -283,8 +283,8 @@ int wd_dslash_resident(wd_op *op, int in_slot, int out_parity, int dagger);
  * that ends each Schur operator of the CGNR iteration (tuned on its own: its
  * register demand differs).  us (optional, n entries) receives the
  * measured microseconds per launch of every candidate (0 for a candidate
- * that was not timed: link staging applies to FP16/BF16 storage only, and
- * entries past the candidate count); block, min_blocks, sites_per_thread and
+ * that was not timed: link staging applies to FP16/BF16 storage only, FP64
+ * hops have one configuration, and entries past the candidate count); block, min_blocks, sites_per_thread and
  * staged (optional; staged = 1: the link records of the eight hops are copied
  * into shared memory at kernel start and the neighbour spinors are loaded two
  * hops ahead; staged = 2: the same with the spinors three hops ahead)

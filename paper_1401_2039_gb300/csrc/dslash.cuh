@@ -1041,9 +1041,9 @@ void launch_any_cfg(int cfg, const DslashArgs<R> &a, cudaStream_t s) {
     }
 }
 
-template <typename S, typename R, int RECON>
-cudaError_t launch_dslash_t(const DslashLaunch &L, cudaStream_t s) {
-    DslashArgs<R> a;
+// Kernel arguments of a launch (an empty site range is not an error).
+template <typename R>
+cudaError_t fill_dslash_args(const DslashLaunch &L, DslashArgs<R> &a) {
     a.g = L.g;
     const int q = 1 - L.out_parity;
     a.gauge_out = (const char *)L.gauge->ptr[L.out_parity];
@@ -1063,11 +1063,18 @@ cudaError_t launch_dslash_t(const DslashLaunch &L, cudaStream_t s) {
     a.h0 = L.h_begin;
     a.h1 = L.h_end < 0 ? L.g.vh : L.h_end;
     if (a.h0 < 0 || a.h1 > L.g.vh || a.h0 > a.h1) return cudaErrorInvalidValue;
+    // the per-warp partials of a fused norm assume a launch over every site
+    if (L.red && (a.h0 != 0 || a.h1 != L.g.vh)) return cudaErrorInvalidValue;
+    return cudaSuccess;
+}
+
+template <typename S, typename R, int RECON>
+cudaError_t launch_dslash_t(const DslashLaunch &L, cudaStream_t s) {
+    DslashArgs<R> a;
+    cudaError_t ea = fill_dslash_args<R>(L, a);
+    if (ea != cudaSuccess) return ea;
     if (a.h1 == a.h0) return cudaSuccess;
     const int cfg = L.cfg;
-    if (L.red) {   // the per-warp partials assume a launch over every site
-        if (a.h0 != 0 || a.h1 != L.g.vh) return cudaErrorInvalidValue;
-    }
     if (L.red) {   // fused norm (after an xpay epilogue), then the fixed-order finish
         if (L.dagger) launch_any_cfg<S, R, RECON, 1, EPI_XPAY, 1>(cfg, a, s);
         else launch_any_cfg<S, R, RECON, 0, EPI_XPAY, 1>(cfg, a, s);

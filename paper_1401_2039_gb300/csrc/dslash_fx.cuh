@@ -1,0 +1,443 @@
+// Hopping term on FP64 fields in block fixed-point integer arithmetic.
+//
+// GB300 issues FP64 at 2 lanes per clock and SM (measured 0.63 T FMA/s against
+// 37 T FP32 FMA/s); 64-bit integer multiply-adds (IMAD.WIDE, 32 x 32 + 64)
+// run at 64.  One site's FP64 hopping term is ~900 FP64 operations and was
+// bound by that pipe: 1673 us at 32^3 x 64, 558 us at 24^3 x 48, 131 us at
+// 16^3 x 32, 55 us at 4^4.  Here the SU(3) products and the sum over the eight
+// hops run on the integer pipes; FP64 keeps the spin projection (12 additions
+// per hop) and the epilogue: 516, 172, 41 and 11 us.  What bounds it now: issue
+// (46 % active at the 20 warps per SM that 96 registers allow), with the FP64
+// pipe 53 % busy and DRAM at 40 %.
+//
+// Numbers.  A link element is u = Fu 2^(eu - 61) with a 61-bit integer Fu and
+// one exponent eu per link: |u| <= 2^eu, and the absolute values of the six
+// reals of any row or column add to at most 2.5 2^eu (0 for every SU(3) link,
+// whose rows add to at most sqrt(6)).  It is stored as two signed limbs, Fu =
+// u1 2^32 + u0, |u1| <= 2^29, |u0| <= 2^31, converted once when the gauge field
+// is loaded.  The projected half-spinor row of a hop (6 reals, FP64) is
+// converted to 60-bit integers Fh = h1 2^32 + h0, |h1| <= 2^28, with one shared
+// exponent.  Then
+//   sum Fu Fh = 2^64 (sum u1 h1 + 2^-32 sum (u1 h0 + u0 h1)) + ...
+// with two 64-bit accumulators per real sum; the omitted u0 h0 terms are below
+// a quarter of the last place each.  |sum (u1 h0 + u0 h1)| <= 2.5 2^60 + 6 2^59
+// < 2^63, |sum u1 h1| <= 2.5 2^57, and the sum over the eight hops (exponent XA
+// of the site's accumulators, raised when a larger hop arrives) stays below
+// 2^62.  The last place of a hop is 2^-57 of twice its largest component: the
+// result is one rounding of a value good to about 2^-56 of the site's scale,
+// where FP64 arithmetic rounds after every operation.  Against 113-bit
+// arithmetic (relative 2-norm, 6 x 10 x 14 x 18): Gaussian fields 7.0e-17 (FP64
+// arithmetic 1.5e-16), fields falling by e^3 per time slice 7.0e-17 (1.4e-16),
+// a point source after two applications of D 5.8e-17 (7.1e-17).
+//
+// Hops whose half spinor is zero contribute nothing.  Infinities, NaN,
+// half spinors below 2^-523 or from 2^477 in magnitude, and links outside
+// 2^-60 .. 2^60 send the site to the plain FP64 hopping term (fx_site_f64).
+#pragma once
+
+#include "dslash.cuh"
+
+namespace wd {
+
+struct FxArgs {
+    DslashArgs<double> d;     // the FP64 links serve the sites that fall back
+    int recon;                // their format
+    int dagger;
+    const char *fx_out, *fx_in;   // fixed-point links: 9 planes (re, im limbs) per direction
+    size_t fx_dir_bytes;
+    const int16_t *ex_out, *ex_in;   // link exponents [direction][stride]
+    const int *any_exp;       // nonzero: some link exponent of the field is not 0
+};
+
+// 2^-523 and 2^477 as biased FP64 exponents: far enough from the ends of the
+// range that no product or sum of a hop leaves it
+constexpr int FX_MIN_EXP = 500, FX_MAX_EXP = 1500;
+constexpr int FX_BAD_EXP = -32768;     // link exponent of a link that cannot be converted
+constexpr int FX_LINK_EXP = 60;
+constexpr int FX_PLANES = 9;
+
+// c + a b, 32 x 32 -> 64 bits signed, as the carry pair that assembles into
+// one IMAD.WIDE (mad.wide.s32 becomes a product and a separate addition, and
+// the C++ expression is reordered across the sums)
+__device__ __forceinline__ long long imadw(int a, int b, long long c) {
+    unsigned lo;
+    int hi;
+    asm("mad.lo.cc.u32 %0, %2, %3, %4;\n\tmadc.hi.s32 %1, %2, %3, %5;"
+        : "=&r"(lo), "=r"(hi)
+        : "r"(a), "r"(b), "r"((unsigned)c), "r"((int)(c >> 32)));
+    return (long long)(((unsigned long long)(unsigned)hi << 32) | lo);
+}
+// arithmetic shift right by min(d, 63), and the logical one (0 from 64 on)
+__device__ __forceinline__ long long sar64(long long v, int d) { return v >> min(d, 63); }
+__device__ __forceinline__ unsigned long long shr64(unsigned long long v, unsigned d) {
+    unsigned long long r;
+    asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(d));
+    return r;
+}
+
+// Fh of the FP64 value v against the block exponent word eh ((E << 20) |
+// 0xFFFFF with E its biased exponent, at least v's): +-(mantissa 2^7) >> (E -
+// e), negated if flip's sign bit is set.  Zeros and values 2^-60 below the
+// block give 0.
+__device__ __forceinline__ long long fx_fixed(double v, unsigned eh, int flip) {
+    const int hi = __double2hiint(v), lo = __double2loint(v);
+    const unsigned s = (eh - (unsigned)(hi & 0x7FFFFFFF)) >> 20;
+    const unsigned m = ((unsigned)hi & 0xFFFFFu) | 0x100000u;
+    unsigned long long x = (((unsigned long long)m << 32) | (unsigned)lo) << 7;
+    x = shr64(x, s);
+    const long long sg = (long long)((hi ^ flip) >> 31);
+    return ((long long)x ^ sg) - sg;
+}
+// the signed limbs of f
+__device__ __forceinline__ void fx_split(long long f, int &l1, int &l0) {
+    l0 = (int)f;
+    l1 = (int)(f >> 32) + (int)((unsigned)l0 >> 31);
+}
+
+// v 2^(x - 1079) rounded to FP64 (x in about 500 .. 1600): the conversion
+// instruction, then the exponent field
+__device__ __forceinline__ double fx_to_double(long long v, int x) {
+    const double d = __ll2double_rn(v);
+    const int hi = __double2hiint(d);
+    return __hiloint2double(v == 0 ? 0 : hi + (x - 1079) * (1 << 20), __double2loint(d));
+}
+
+// H in at one site in FP64 arithmetic (the generic hop): the sites that the
+// fixed-point form does not cover
+template <int RECON, int DAG>
+__device__ __noinline__ void fx_site_f64(const DslashArgs<double> &a, long h, double *acc) {
+    int c[4];
+    site_coords(a.g, h, a.parity, c);
+    for (int k = 0; k < 24; ++k) acc[k] = 0;
+    hop_pair<double, double, RECON, 0, DAG>(a, c, h, acc);
+    hop_pair<double, double, RECON, 1, DAG>(a, c, h, acc);
+    hop_pair<double, double, RECON, 2, DAG>(a, c, h, acc);
+    hop_pair<double, double, RECON, 3, DAG>(a, c, h, acc);
+}
+
+__device__ __forceinline__ double2 ld_nc_d2(const char *p) {
+    const uint4 v = ld_nc_v4(p);
+    return make_double2(__hiloint2double((int)v.y, (int)v.x), __hiloint2double((int)v.w, (int)v.z));
+}
+
+// neighbour of site h in direction mu, forward or backward
+__device__ __forceinline__ unsigned fx_neighbour(const Geom &g, unsigned h, const int c[4], int mu,
+                                                 bool fwd, bool &wrap) {
+    if (mu == 0) {
+        int xn = fwd ? c[0] + 1 : c[0] - 1;
+        wrap = fwd ? xn == g.L[0] : xn < 0;
+        if (wrap) xn = fwd ? 0 : g.L[0] - 1;
+        return h + (unsigned)((xn >> 1) - (c[0] >> 1));
+    }
+    const int cm = mu == 1 ? c[1] : mu == 2 ? c[2] : c[3];
+    const unsigned step = g.step[mu], back = g.back[mu];
+    wrap = cm == (fwd ? g.L[mu] - 1 : 0);
+    return fwd ? (wrap ? h - back : h + step) : (wrap ? h + back : h - step);
+}
+
+// The hops run as a loop over one body: mu, the sense and the row are the same
+// for a warp, so every choice on them is a uniform branch (unrolled by
+// direction and sense, warps waited on instruction fetch: 2.4 stalled cycles
+// per instruction).
+
+// the nine link elements of the hop from site `site`, in the order of the
+// product: U forward, its transpose backward (32-bit byte offsets from a
+// warp-uniform base)
+__device__ __forceinline__ void fx_links(const FxArgs &A, unsigned site, int mu, bool fwd,
+                                         uint4 U[3][3]) {
+    const size_t plane = (size_t)A.d.g.stride * 16;
+    const char *pu = (fwd ? A.fx_out : A.fx_in) + mu * A.fx_dir_bytes;
+    const size_t pi = (fwd ? 3 : 1) * plane, pj = (fwd ? 1 : 3) * plane;
+    const unsigned o = site * 16u;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) U[i][j] = ld_stream_v4(pu + i * pi + j * pj + o);
+}
+
+// whether row k enters gamma_mu with a minus sign: row 0 of gamma_y, row 1 of
+// gamma_z
+__device__ __forceinline__ bool fx_row_neg(int mu, int k) {
+    return mu == 1 ? k == 0 : mu == 2 && k == 1;
+}
+
+// row k of the half spinor at neighbour hn, [colour][re, im]: p_k + s (i) q with
+// the partner spin q = 3 - k (x, y) or 2 + k (z, t)
+__device__ __forceinline__ void fx_half_row(const FxArgs &A, unsigned hn, int mu, int k, bool fwd,
+                                            double r[6]) {
+    const size_t plane = (size_t)A.d.g.stride * 16;
+    const char *pp = (const char *)A.d.in + k * plane;
+    const char *pq = (const char *)A.d.in + (mu < 2 ? 3 - k : 2 + k) * plane;
+    const unsigned o = hn * 16u;
+    const bool neg = (fwd != (A.dagger != 0)) != fx_row_neg(mu, k);
+    const double s = __hiloint2double(neg ? (int)0xBFF00000u : 0x3FF00000, 0);
+    const double ns = __hiloint2double(neg ? 0x3FF00000 : (int)0xBFF00000u, 0);
+    double2 p[3], q[3];
+#pragma unroll
+    for (int cc = 0; cc < 3; ++cc) {
+        p[cc] = ld_nc_d2(pp + (4 * cc) * plane + o);
+        q[cc] = ld_nc_d2(pq + (4 * cc) * plane + o);
+    }
+    if ((mu & 1) == 0) {   // p + s i q
+#pragma unroll
+        for (int cc = 0; cc < 3; ++cc) {
+            r[2 * cc] = fma(ns, q[cc].y, p[cc].x);
+            r[2 * cc + 1] = fma(s, q[cc].x, p[cc].y);
+        }
+    } else {               // p + s q
+#pragma unroll
+        for (int cc = 0; cc < 3; ++cc) {
+            r[2 * cc] = fma(s, q[cc].x, p[cc].x);
+            r[2 * cc + 1] = fma(s, q[cc].y, p[cc].y);
+        }
+    }
+}
+
+// r *= the boundary phase of direction mu (it commutes with the link)
+__device__ __forceinline__ void fx_phase(const FxArgs &A, int mu, bool fwd, double r[6]) {
+    const double pr = A.d.ph[2 * mu], pi = fwd ? A.d.ph[2 * mu + 1] : -A.d.ph[2 * mu + 1];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const double t = r[2 * i] * pr - r[2 * i + 1] * pi;
+        r[2 * i + 1] = r[2 * i] * pi + r[2 * i + 1] * pr;
+        r[2 * i] = t;
+    }
+}
+
+// any bit of r but the signs set (bits, not values: FP64 comparisons would
+// cost as much as the sums)
+__device__ __forceinline__ unsigned fx_bits(const double r[6]) {
+    unsigned any = 0;
+#pragma unroll
+    for (int i = 0; i < 6; ++i)
+        any |= ((unsigned)__double2hiint(r[i]) & 0x7FFFFFFFu) | (unsigned)__double2loint(r[i]);
+    return any;
+}
+__device__ __forceinline__ unsigned fx_max(const double r[6]) {
+    unsigned mx = 0;
+#pragma unroll
+    for (int i = 0; i < 6; ++i) mx = max(mx, (unsigned)__double2hiint(r[i]) & 0x7FFFFFFFu);
+    return mx;
+}
+
+// the row transported, u[colour][re, im], in units of the block exponent eh
+__device__ __forceinline__ void fx_product(const uint4 U[3][3], const double r[6], unsigned eh,
+                                           bool fwd, long long u[6]) {
+    // backward: conj(U)^T h = conj(U^T conj(h)); i are the limbs of the
+    // imaginary parts entering the product, j those of their negatives
+    const int cj = fwd ? 0 : (int)0x80000000u;
+    int r1[3], r0[3], i1[3], i0[3], j1[3], j0[3];
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        const long long re = fx_fixed(r[2 * b], eh, 0), im = fx_fixed(r[2 * b + 1], eh, cj);
+        fx_split(re, r1[b], r0[b]);
+        fx_split(im, i1[b], i0[b]);
+        fx_split(-im, j1[b], j0[b]);
+    }
+    // the leading and the middle sums of the real and the imaginary part; the
+    // middle ones start at half a last place
+    long long ph[3], pm[3], qh[3], qm[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        ph[i] = qh[i] = 0;
+        pm[i] = qm[i] = 1ll << 31;
+    }
+#pragma unroll
+    for (int b = 0; b < 3; ++b)
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const int u1r = (int)U[i][b].y, u0r = (int)U[i][b].x;
+            const int u1i = (int)U[i][b].w, u0i = (int)U[i][b].z;
+            ph[i] = imadw(u1r, r1[b], ph[i]);
+            pm[i] = imadw(u1r, r0[b], pm[i]);
+            qh[i] = imadw(u1r, i1[b], qh[i]);
+            qm[i] = imadw(u1r, i0[b], qm[i]);
+            pm[i] = imadw(u0r, r1[b], pm[i]);
+            qm[i] = imadw(u0r, i1[b], qm[i]);
+            ph[i] = imadw(u1i, j1[b], ph[i]);
+            pm[i] = imadw(u1i, j0[b], pm[i]);
+            qh[i] = imadw(u1i, r1[b], qh[i]);
+            qm[i] = imadw(u1i, r0[b], qm[i]);
+            pm[i] = imadw(u0i, j1[b], pm[i]);
+            qm[i] = imadw(u0i, r1[b], qm[i]);
+        }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        u[2 * i] = imadw((int)(pm[i] >> 32), 1, ph[i]);
+        u[2 * i + 1] = imadw((int)(qm[i] >> 32), 1, qh[i]);
+    }
+    if (!fwd) {
+#pragma unroll
+        for (int i = 0; i < 3; ++i) u[2 * i + 1] = -u[2 * i + 1];
+    }
+}
+
+// a += u, and the row's term of spin 2 or 3 without the projector's sign, b +=
+// -i u (x, z) or u (y, t), subtracted if minus
+__device__ __forceinline__ void fx_accumulate(long long a[6], long long b[6], const long long u[6],
+                                              int mu, bool minus) {
+#pragma unroll
+    for (int i = 0; i < 6; ++i) a[i] += u[i];
+    if ((mu & 1) == 0) {
+        if (minus) {
+#pragma unroll
+            for (int i = 0; i < 3; ++i) { b[2 * i] -= u[2 * i + 1]; b[2 * i + 1] += u[2 * i]; }
+        } else {
+#pragma unroll
+            for (int i = 0; i < 3; ++i) { b[2 * i] += u[2 * i + 1]; b[2 * i + 1] -= u[2 * i]; }
+        }
+    } else if (minus) {
+#pragma unroll
+        for (int i = 0; i < 6; ++i) b[i] -= u[i];
+    } else {
+#pragma unroll
+        for (int i = 0; i < 6; ++i) b[i] += u[i];
+    }
+}
+
+__device__ __forceinline__ bool fx_out_of_range(int eb, int eu) {
+    return eb < FX_MIN_EXP || eb > FX_MAX_EXP || eu == FX_BAD_EXP;
+}
+__device__ __forceinline__ int fx_link_exp(const FxArgs &A, bool any_exp, unsigned site, int mu,
+                                           bool fwd) {
+    if (!any_exp) return 0;
+    return (fwd ? A.ex_out : A.ex_in)[(size_t)mu * A.d.g.stride + site];
+}
+// the vote makes this a branch (as predicated instructions the FP64 products
+// of the phase would take the pipe in every hop)
+__device__ __forceinline__ bool fx_wraps(const FxArgs &A, int mu, bool wrap) {
+    return (A.d.phase_on >> mu & 1u) && __any_sync(__activemask(), wrap) && wrap;
+}
+
+// the site by the plain FP64 hop
+__device__ __forceinline__ void fx_fallback(const FxArgs &A, unsigned h, double t[24]) {
+    if (A.recon == 12) {
+        if (A.dagger) fx_site_f64<12, 1>(A.d, h, t);
+        else fx_site_f64<12, 0>(A.d, h, t);
+    } else {
+        if (A.dagger) fx_site_f64<18, 1>(A.d, h, t);
+        else fx_site_f64<18, 0>(A.d, h, t);
+    }
+}
+
+// Work split: the four warps of a 128-thread block take 32 consecutive sites,
+// warp (k, dir) row k of the half spinors of their four forward or four
+// backward hops.  One thread per site needs 24 64-bit accumulators (152
+// registers, 12 warps per SM); it measured the same at 32^3 x 64 (518 against
+// 515 us) and loses below: 188 / 172 us at 24^3 x 48, 48 / 41 at 16^3 x 32, 24 /
+// 11 at 8^4.  Row k goes into
+// spin k (accumulator a) and spin 3 - k for directions x and y, 2 + k for z
+// and t (accumulator b, exchanged between the two rows' warps in between); the
+// forward and the backward warp add up at the end, where one keeps spin k and
+// the other spin 2 + k.  Both exchanges go through shared memory.
+constexpr int FX_BLOCK = 128;
+constexpr int FX_SITES = 32;      // sites per block
+
+struct FxShared {
+    long long v[2][4][6][32];
+    int xa[2][4][32];
+};
+
+// every thread of the block calls it, the four warps of one lane on the same
+// site h: v = spin k (forward warps) or 2 + k of H in, [colour][re, im]
+__device__ __forceinline__ void fx_site(const FxArgs &A, unsigned h, int w, FxShared &sh,
+                                             double v[6]) {
+    const int lane = threadIdx.x & 31, k = w & 1;
+    const bool fwd = w < 2;
+    int c[4];
+    site_coords(A.d.g, h, A.d.parity, c);
+    const bool any_exp = __ldg(A.any_exp) != 0;
+    long long a[6], b[6];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) a[i] = b[i] = 0;
+    int xa = -(1 << 20);
+    bool bad = false;
+#pragma unroll 1
+    for (int mu = 0; mu < 4; ++mu) {
+        if (mu == 2) {   // row k goes on with spin 2 + k
+#pragma unroll
+            for (int i = 0; i < 6; ++i) sh.v[0][w][i][lane] = b[i];
+            sh.xa[0][w][lane] = xa;
+            __syncwarp();
+            __syncthreads();
+            const int xo = sh.xa[0][w ^ 1][lane];
+#pragma unroll
+            for (int i = 0; i < 6; ++i) b[i] = sh.v[0][w ^ 1][i][lane];
+            if (xo != xa) {   // b comes in the other row's units
+                const int x = max(xo, xa);
+                if (xa >= 0) {
+#pragma unroll
+                    for (int i = 0; i < 6; ++i) a[i] = sar64(a[i], x - xa);
+                }
+                if (xo >= 0) {
+#pragma unroll
+                    for (int i = 0; i < 6; ++i) b[i] = sar64(b[i], x - xo);
+                }
+                xa = x;
+            }
+        }
+        bool wrap;
+        const unsigned hn = fx_neighbour(A.d.g, h, c, mu, fwd, wrap), site = fwd ? h : hn;
+        uint4 U[3][3];
+        fx_links(A, site, mu, fwd, U);
+        const int eu = fx_link_exp(A, any_exp, site, mu, fwd);
+        double r[6];
+        fx_half_row(A, hn, mu, k, fwd, r);
+        if (fx_wraps(A, mu, wrap)) fx_phase(A, mu, fwd, r);
+        const int eb = (int)(fx_max(r) >> 20);
+        if (fx_out_of_range(eb, eu)) {
+            if (fx_bits(r) != 0 || eu == FX_BAD_EXP) bad = true;
+            continue;
+        }
+        if (eb + eu > xa) {   // a larger hop
+            const int x = eb + eu;
+            if (xa >= 0) {
+                const int d = x - xa;
+#pragma unroll
+                for (int i = 0; i < 6; ++i) {
+                    a[i] = sar64(a[i], d);
+                    b[i] = sar64(b[i], d);
+                }
+            }
+            xa = x;
+        }
+        long long u[6];
+        fx_product(U, r, ((unsigned)(xa - eu) << 20) | 0xFFFFFu, fwd, u);
+        fx_accumulate(a, b, u, mu, fx_row_neg(mu, k));
+    }
+    // the forward warp keeps a and gives b, the backward warp the reverse; a
+    // bad site is marked in the exponent
+#pragma unroll
+    for (int i = 0; i < 6; ++i) sh.v[1][w][i][lane] = fwd ? b[i] : a[i];
+    sh.xa[1][w][lane] = bad ? (1 << 24) : xa;
+    __syncwarp();
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) bad = bad || sh.xa[1][q][lane] == (1 << 24);
+    if (bad) {
+        double t[24];
+        fx_fallback(A, h, t);
+        const int sp = fwd ? k : 2 + k;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            v[2 * i] = t[8 * i + 2 * sp];
+            v[2 * i + 1] = t[8 * i + 2 * sp + 1];
+        }
+        return;
+    }
+    const int xb = sh.xa[1][w ^ 2][lane], xm = max(xa, xb);
+    // opposite projectors: spins 2, 3 take forward minus backward, times the
+    // forward one's sign (-1 for H, +1 for H^dag)
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+        long long got = sh.v[1][w ^ 2][i][lane], own = fwd ? a[i] : b[i];
+        if (xa != xb) {
+            got = xb >= 0 ? sar64(got, xm - xb) : 0;
+            own = xa >= 0 ? sar64(own, xm - xa) : 0;
+        }
+        const long long sum = fwd ? own + got : A.dagger ? got - own : own - got;
+        v[i] = fx_to_double(sum, xm);
+    }
+}
+
+}  // namespace wd

@@ -570,6 +570,13 @@ struct GaugeSet {       // links of both parities, one precision/reconstruction
     size_t dir_bytes = 0;               // bytes of one direction block
     int prec = WD_F64;
     int recon = 18;
+    // FP64 links as fixed-point limbs for the integer hop (dslash_fx.cuh):
+    // [parity] -> 4 direction blocks of 9 planes, the link exponents
+    // [direction][stride], and whether any exponent is not 0.  Null: none kept.
+    void *fx[2] = {nullptr, nullptr};
+    size_t fx_dir_bytes = 0;
+    int16_t *fx_exp[2] = {nullptr, nullptr};
+    int *any_exp = nullptr;
 };
 
 enum Epilogue { EPI_PLAIN = 0, EPI_XPAY = 1 };
@@ -606,6 +613,11 @@ inline unsigned phase_mask(const double phase[8]) {
 
 // dslash.cu
 cudaError_t launch_dslash(const DslashLaunch &L, int prec, cudaStream_t s);
+
+// dslash_fx.cu: the FP64 hop in fixed-point arithmetic (L.gauge->fx set), and
+// the fixed-point copy of a gauge set's FP64 links
+cudaError_t launch_dslash_fx(const DslashLaunch &L, cudaStream_t s);
+cudaError_t launch_gauge_fx(const GaugeSet &gs, const Geom &g, cudaStream_t s);
 
 // blas.cu
 // r -= alpha Ap and ||r||^2; then, next iteration, x += alpha_x p and
