@@ -288,7 +288,8 @@ int wd_dslash_resident(wd_op *op, int in_slot, int out_parity, int dagger);
  * staged (optional; staged = 1: the link records of the eight hops are copied
  * into shared memory at kernel start and the neighbour spinors are loaded two
  * hops ahead; staged = 2: the same with the spinors three hops ahead)
- * describe the chosen one.  Returns its
+ * describe the chosen one; candidate 8 (FP32, FP16, BF16) runs one warp per hop,
+ * 32 sites per block of 256 threads.  Returns its
  * index, or -1 for a null handle.  Setting WD_DSLASH_CFG=k in the
  * environment forces candidate k, WD_TUNE=0 keeps candidate 0. */
 int wd_dslash_tuning(const wd_op *op, int hi, double *us, int n, int *block, int *min_blocks,

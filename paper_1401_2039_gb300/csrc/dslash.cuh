@@ -400,6 +400,27 @@ __device__ __forceinline__ void hop_pair(const DslashArgs<R> &a, const int c[4],
     }
 }
 
+// u = hop (MU, DIR), transported and with its phase (FP32 arithmetic), as in
+// hop_pair
+template <typename S, int RECON, int MU, int DIR, int DAG>
+__device__ __forceinline__ void transport_f32(const DslashArgs<float> &a, const int c[4], long h,
+                                              cx<float> u[2][3]) {
+    constexpr int SF = DAG ? +1 : -1;
+    bool wrap;
+    const long hn = neighbour<MU, DIR>(a.g, h, c, wrap);
+    float psi[24];
+    Rec<S, 24>::template load<float, 0>(a.in, a.g.stride, hn, psi);
+    float U[18];
+    load_link<S, float, RECON>((DIR > 0 ? a.gauge_out : a.gauge_in) + MU * a.dir_bytes, a.g.stride,
+                               DIR > 0 ? h : hn, U);
+    cx<float> hs[2][3];
+    project<MU, (DIR > 0 ? SF : -SF)>(psi, hs);
+    if (DIR > 0) su3_mul(U, hs, u);
+    else su3_adj_mul(U, hs, u);
+    if (wrap && (a.phase_on >> MU & 1u))
+        phase_mul(u, a.ph[2 * MU], DIR > 0 ? a.ph[2 * MU + 1] : -a.ph[2 * MU + 1]);
+}
+
 // ------------------------------------------------------ FP16 and BF16 storage
 // With 16-bit storage the generic hop spends about a sixth of its
 // instructions converting elements to FP32 (one conversion per stored
@@ -705,11 +726,11 @@ __device__ __forceinline__ void load_link_words(const DslashArgs<float> &a, unsi
     }
 }
 
-// acc += hop (MU, DIR) of the neighbour words p with the link words U
-// (12-real records: words 0..5, row 2 rebuilt here)
+// u = hop (MU, DIR), transported and with its phase, of the neighbour words p
+// with the link words U (12-real records: words 0..5, row 2 rebuilt here)
 template <typename HT, int RECON, int MU, int DIR, int DAG>
-__device__ __forceinline__ void compute_hop_h2(const DslashArgs<float> &a, const uint32_t p[12],
-                                               bool wrap, uint32_t U[9], float *acc) {
+__device__ __forceinline__ void transport_h2(const DslashArgs<float> &a, const uint32_t p[12],
+                                             bool wrap, uint32_t U[9], cx<float> u[2][3]) {
     constexpr int SF = DAG ? +1 : -1;
     constexpr int S = DIR > 0 ? SF : -SF;
     if (RECON == 12) {
@@ -731,14 +752,22 @@ __device__ __forceinline__ void compute_hop_h2(const DslashArgs<float> &a, const
     }
     uint32_t hs[2][3];
     project_h2<HT, MU, S>(p, hs);
-    cx<float> u[2][3];
     if (DIR > 0) su3_mul_h2<HT>(U, hs, u);
     else su3_adj_mul_h2<HT>(U, hs, u);
     if (wrap && (a.phase_on >> MU & 1u)) {   // a phase of exactly 1 is skipped
         const float pr = (float)a.ph[2 * MU], pi = (float)a.ph[2 * MU + 1];
         phase_mul(u, pr, DIR > 0 ? pi : -pi);
     }
-    accumulate_x2<MU, S>(acc, u);
+}
+
+// acc += the same
+template <typename HT, int RECON, int MU, int DIR, int DAG>
+__device__ __forceinline__ void compute_hop_h2(const DslashArgs<float> &a, const uint32_t p[12],
+                                               bool wrap, uint32_t U[9], float *acc) {
+    constexpr int SF = DAG ? +1 : -1;
+    cx<float> u[2][3];
+    transport_h2<HT, RECON, MU, DIR, DAG>(a, p, wrap, U, u);
+    accumulate_x2<MU, (DIR > 0 ? SF : -SF)>(acc, u);
 }
 
 // ---- pipelined: spinor and link words of the next hop in registers
@@ -993,17 +1022,173 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_dslash(const DslashArgs<R> a) {
     if (NORM) warp_partials<BLOCK, SPT>(nrm, a.g.vh, a.red.partials);
 }
 
+// ---- one warp per hop
+// One thread per site does a site's eight hops one after the other; small and
+// medium lattices give an SM few such threads, and the hop is then latency
+// alone.  Here a block of eight warps takes 32 consecutive sites, warp w hop w
+// of all of them; the transported half spinors meet in shared memory, and one
+// warp per 16-byte plane of the output record adds the eight contributions in
+// hop order, with the same FP32 additions, products and epilogue as k_dslash:
+// bitwise its result, so the tuner may choose between them freely.  It needs
+// 56 registers (32 warps per SM; at 48 registers the same within 5 %).  Plain
+// hop, best other candidate -> this one, launches back to back:
+//   FP32/18  32^3 x 64 137.9 -> 130.9 us, 24^3 x 48 48.3 -> 43.8, 16^3 x 32 16.4
+//            -> 12.7, 12^3 x 24 8.2 -> 6.9, 8^4 6.5 -> 4.2, 4^4 6.2 -> 4.2
+//   FP16/18  24^3 x 48 27.7 -> 26.9, 12^3 x 24 6.2 -> 5.7, 8^4 4.8 -> 4.5;
+//            FP16/12 12^3 x 24 6.3 -> 6.1, 8^4 5.8 -> 4.4; above that the
+//            staged 16-bit candidates are faster (32^3 x 64 FP16/12 55.7 against
+//            83.1: the exchange through shared memory moves FP32).
+constexpr int SPLIT_SITES = 32;
+constexpr int SPLIT_BLOCK = 256;
+
+struct SplitStage {
+    float2 u[8][6][SPLIT_SITES];   // [hop][3 row + colour][site]
+    float o[24][SPLIT_SITES];      // outputs before rounding (fused norm)
+};
+
+template <typename S, int RECON, int DAG, int I>
+__device__ __forceinline__ void split_hop(const DslashArgs<float> &a, const int c[4], long h,
+                                          SplitStage &st) {
+    constexpr int MU = I / 2, DIR = (I & 1) ? -1 : +1;
+    cx<float> u[2][3];
+    if constexpr (packed16<S>()) {
+        HopH2 d;
+        load_hop_h2<RECON, I>(a, c, (unsigned)h, d);
+        transport_h2<S, RECON, MU, DIR, DAG>(a, d.s.p, d.s.wrap, d.U, u);
+    } else {
+        transport_f32<S, RECON, MU, DIR, DAG>(a, c, h, u);
+    }
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) st.u[I][3 * k + q][lane] = make_float2(u[k][q].re, u[k][q].im);
+}
+
+// v (re, im) += the term of spin SP, colour col of hop I: accumulate<MU, SGN>
+template <int DAG, int I, int SP>
+__device__ __forceinline__ void split_add(const SplitStage &st, int col, int lane, float &re,
+                                          float &im) {
+    constexpr int MU = I / 2;
+    constexpr int SGN = ((I & 1) == 0) == (DAG != 0) ? +1 : -1;
+    // the row that enters, and its factor: 0 u, 1 -u, 2 i u, 3 -i u
+    constexpr int ROW = SP < 2 ? SP : MU < 2 ? 3 - SP : SP - 2;
+    constexpr int F = SP < 2 ? 0
+                      : MU == 0 ? (SGN > 0 ? 3 : 2)
+                      : MU == 1 ? ((SP == 2) == (SGN > 0) ? 0 : 1)
+                      : MU == 2 ? ((SP == 2) == (SGN > 0) ? 3 : 2)
+                                : (SGN > 0 ? 0 : 1);
+    const float2 u = st.u[I][3 * ROW + col][lane];
+    if (F == 0) { re += u.x; im += u.y; }
+    else if (F == 1) { re -= u.x; im -= u.y; }
+    else if (F == 2) { re -= u.y; im += u.x; }
+    else { re += u.y; im -= u.x; }
+}
+
+template <int DAG, int SP>
+__device__ __forceinline__ void split_sum(const SplitStage &st, int col, int lane, float &re,
+                                          float &im) {
+    re = im = 0.0f;
+    split_add<DAG, 0, SP>(st, col, lane, re, im);
+    split_add<DAG, 1, SP>(st, col, lane, re, im);
+    split_add<DAG, 2, SP>(st, col, lane, re, im);
+    split_add<DAG, 3, SP>(st, col, lane, re, im);
+    split_add<DAG, 4, SP>(st, col, lane, re, im);
+    split_add<DAG, 5, SP>(st, col, lane, re, im);
+    split_add<DAG, 6, SP>(st, col, lane, re, im);
+    split_add<DAG, 7, SP>(st, col, lane, re, im);
+}
+
+template <typename S, int RECON, int DAG, int EPI, int NORM, int MINB>
+__global__ void __launch_bounds__(SPLIT_BLOCK, MINB)
+k_dslash_split(const __grid_constant__ DslashArgs<float> a) {
+    __shared__ SplitStage st;
+    const int lane = threadIdx.x & 31, w = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);
+    const long hs = a.h0 + (long)blockIdx.x * SPLIT_SITES + lane;
+    const long h = hs < a.h1 ? hs : a.h1 - 1;
+    int c[4];
+    site_coords(a.g, h, a.parity, c);
+    switch (w) {
+    case 0: split_hop<S, RECON, DAG, 0>(a, c, h, st); break;
+    case 1: split_hop<S, RECON, DAG, 1>(a, c, h, st); break;
+    case 2: split_hop<S, RECON, DAG, 2>(a, c, h, st); break;
+    case 3: split_hop<S, RECON, DAG, 3>(a, c, h, st); break;
+    case 4: split_hop<S, RECON, DAG, 4>(a, c, h, st); break;
+    case 5: split_hop<S, RECON, DAG, 5>(a, c, h, st); break;
+    case 6: split_hop<S, RECON, DAG, 6>(a, c, h, st); break;
+    default: split_hop<S, RECON, DAG, 7>(a, c, h, st); break;
+    }
+    __syncthreads();
+    // one plane of K reals per warp: colour j K / 8, spins from (j K / 2) % 4
+    constexpr int K = 16 / (int)sizeof(S), PLANES = 24 / K;
+    static_assert(PLANES <= 8, "a warp per plane");
+    if (w < PLANES) {
+        const int j = w, col = j * K / 8;
+        float acc[K];
+        if (K == 8) {
+            split_sum<DAG, 0>(st, col, lane, acc[0], acc[1]);
+            split_sum<DAG, 1>(st, col, lane, acc[2], acc[3]);
+            split_sum<DAG, 2>(st, col, lane, acc[K - 4], acc[K - 3]);
+            split_sum<DAG, 3>(st, col, lane, acc[K - 2], acc[K - 1]);
+        } else if ((j & 1) == 0) {
+            split_sum<DAG, 0>(st, col, lane, acc[0], acc[1]);
+            split_sum<DAG, 1>(st, col, lane, acc[2], acc[3]);
+        } else {
+            split_sum<DAG, 2>(st, col, lane, acc[0], acc[1]);
+            split_sum<DAG, 3>(st, col, lane, acc[2], acc[3]);
+        }
+        float ov[K];
+        if (EPI == EPI_XPAY) {
+            float xv[K];
+            const uint4 x = ld_nc_v4((const char *)a.x + ((long)j * a.g.stride + h) * 16);
+            const uint32_t ww[4] = {x.x, x.y, x.z, x.w};
+            Words<S, float>::unpack(ww, xv, K);
+            if (a.twist_on) twist_reals<K>(xv, j * K, a.twist);
+#pragma unroll
+            for (int t = 0; t < K; t += 2)
+                scale_add_x2(ov[t], ov[t + 1], acc[t], acc[t + 1], a.scale, xv[t], xv[t + 1]);
+        } else {
+#pragma unroll
+            for (int t = 0; t < K; t += 2)
+                scale_x2(ov[t], ov[t + 1], acc[t], acc[t + 1], a.scale);
+            if (a.twist_on) twist_reals<K>(ov, j * K, -a.twist);
+        }
+        if (hs < a.h1) {
+            uint32_t ow[4];
+            Words<S, float>::pack(ov, ow, K);
+            st_v4((char *)a.out + ((long)j * a.g.stride + h) * 16,
+                  make_uint4(ow[0], ow[1], ow[2], ow[3]));
+        }
+        if (NORM) {
+#pragma unroll
+            for (int t = 0; t < K; ++t) st.o[j * K + t][lane] = ov[t];
+        }
+    }
+    if (NORM) {   // the chains of squares of k_dslash, one partial per 32 sites
+        __syncthreads();
+        if (w == 0) {
+            float sq = 0, sq1 = 0;
+#pragma unroll
+            for (int t = 0; t < 24; t += 2) sq_acc_x2(sq, sq1, st.o[t][lane], st.o[t + 1][lane]);
+            const df64 s = warp_sum(hs < a.h1 ? to_df(sq + sq1) : df64(0.0f, 0.0f));
+            if (lane == 0) a.red.partials[blockIdx.x] = s;
+        }
+    }
+}
+
 // Launch configurations the tuner chooses from: threads per block, the
 // minimum resident blocks per SM handed to the register allocator, output
 // sites per thread, and (16-bit storage only) links staged in shared memory
 // with the neighbour spinors two (stage 1) or three (stage 2) hops ahead.
 // A fused norm adds in the same order under every configuration
 // (warp_partials), so every variant can take its own tuned one.
-struct DslashCfg { int block, minb, spt, stage; };
-constexpr int N_DSLASH_CFG = 8;
+// split = 1: one warp per hop (k_dslash_split).
+struct DslashCfg { int block, minb, spt, stage, split = 0; };
+constexpr int N_DSLASH_CFG = 9;
 constexpr DslashCfg DSLASH_CFGS[N_DSLASH_CFG] = {
     {128, 1, 1, 0}, {128, 8, 1, 0}, {128, 6, 1, 0}, {256, 4, 1, 0},
-    {128, 1, 2, 0}, {128, 5, 1, 2}, {128, 6, 1, 1}, {128, 6, 1, 2}};
+    {128, 1, 2, 0}, {128, 5, 1, 2}, {128, 6, 1, 1}, {128, 6, 1, 2},
+    {SPLIT_BLOCK, 3, 1, 0, 1}};
 // whether candidate k is distinct for storage precision prec (staging
 // applies to 16-bit storage only; elsewhere it repeats an unstaged entry)
 inline bool dslash_cfg_applies(int k, int prec) {
@@ -1021,6 +1206,11 @@ constexpr DslashCfg DSLASH_DF_CFGS[N_DSLASH_DF_CFG] = {
 template <typename S, typename R, int RECON, int DAG, int EPI, int NORM, int CFG>
 void launch_cfg(const DslashArgs<R> &a, cudaStream_t s) {
     constexpr DslashCfg C = DSLASH_CFGS[CFG];
+    if constexpr (C.split) {
+        const unsigned grid = (unsigned)((a.h1 - a.h0 + SPLIT_SITES - 1) / SPLIT_SITES);
+        k_dslash_split<S, RECON, DAG, EPI, NORM, C.minb><<<grid, C.block, 0, s>>>(a);
+        return;
+    }
     constexpr int STAGE = packed16<S>() ? C.stage : 0;
     const long per_block = (long)C.block * C.spt;
     const unsigned grid = (unsigned)((a.h1 - a.h0 + per_block - 1) / per_block);
@@ -1037,6 +1227,9 @@ void launch_any_cfg(int cfg, const DslashArgs<R> &a, cudaStream_t s) {
     case 5: launch_cfg<S, R, RECON, DAG, EPI, NORM, 5>(a, s); break;
     case 6: launch_cfg<S, R, RECON, DAG, EPI, NORM, 6>(a, s); break;
     case 7: launch_cfg<S, R, RECON, DAG, EPI, NORM, 7>(a, s); break;
+    case 8:
+        if constexpr (sizeof(S) <= 4) launch_cfg<S, R, RECON, DAG, EPI, NORM, 8>(a, s);
+        break;
     default: launch_cfg<S, R, RECON, DAG, EPI, NORM, 0>(a, s); break;
     }
 }

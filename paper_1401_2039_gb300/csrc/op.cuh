@@ -89,7 +89,7 @@ struct wd_op {
     // tuned launch configuration of the hopping term: [0] storage precision,
     // [1] residual arithmetic, [2] storage precision with xpay and fused norm
     int cfg[3] = {0, 0, 0};
-    double tune_us[3][8] = {};
+    double tune_us[3][wd::N_DSLASH_CFG] = {};
     cudaEvent_t ev_t0 = nullptr, ev_t1 = nullptr;
 
     // CUDA graphs of 2^k CGNR iterations, per solved parity

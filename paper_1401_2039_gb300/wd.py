@@ -21,6 +21,8 @@ WD_OK, WD_ERR_ARG, WD_ERR_DIMS, WD_ERR_CUDA, WD_ERR_NOMEM = 0, 1, 2, 3, 4
 WD_ERR_NOT_CONVERGED, WD_ERR_BREAKDOWN, WD_ERR_TIMEOUT, WD_ERR_STATE = 5, 6, 7, 8
 PRECISIONS = {"f64": 0, "f32": 1, "f16": 2, "bf16": 3}
 RECOVERY = {"reliable": 0, "defect": 1}
+# launch candidates of the single-system hop (wd_dslash_tuning)
+DSLASH_CANDIDATES = 9
 # launch candidates of the batched hop (include/wd.h, wd_batch_tuning): the
 # ones from BATCH_PAIR_FIRST on take two right-hand sides per thread
 BATCH_CANDIDATES = 9
@@ -288,10 +290,10 @@ class WilsonDirac:
         timings (us): storage precision (default), residual arithmetic
         (hi=True), or the storage-precision variant with xpay and fused norm
         (norm=True)."""
-        us = (ctypes.c_double * 8)()
+        us = (ctypes.c_double * DSLASH_CANDIDATES)()
         blk, mb, spt, stg = ctypes.c_int(), ctypes.c_int(), ctypes.c_int(), ctypes.c_int()
         variant = 2 if norm else int(bool(hi))
-        k = self.lib.wd_dslash_tuning(self.handle, variant, us, 8, ctypes.byref(blk),
+        k = self.lib.wd_dslash_tuning(self.handle, variant, us, DSLASH_CANDIDATES, ctypes.byref(blk),
                                       ctypes.byref(mb), ctypes.byref(spt), ctypes.byref(stg))
         return {"index": k, "block": blk.value, "min_blocks": mb.value,
                 "sites_per_thread": spt.value, "staged": bool(stg.value), "stage": stg.value,
