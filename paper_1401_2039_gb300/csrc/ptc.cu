@@ -179,6 +179,21 @@ __global__ void k_ptc_weights(int cout, int cin, const float2 *__restrict__ W,
     B[(long)(N + n) * ldb + K + kk] = __float2bfloat16_rn(w.x);    // Im out <- Im in:  Wr
 }
 
+// The weights of a layer with 16 input channels as the fused kernel's
+// shared-memory images: chunk q = (transport k, channel group), rows n < N, 64
+// columns (re: k 64 + grp 32 + 0..31, im: 576 + the same), in the K-major
+// core-matrix layout (8 rows x 16 bytes contiguous).
+__global__ void k_ptc_weights_fused(int N, const __nv_bfloat16 *__restrict__ B, int ldb,
+                                    __nv_bfloat16 *__restrict__ img) {
+    const long i = (long)blockIdx.x * PTC_BLOCK + threadIdx.x;   // (q, row, column)
+    if (i >= (long)PF_NCHUNK * N * 64) return;
+    const int q = (int)(i / (N * 64)), r = (int)(i - (long)q * N * 64);
+    const int row = r >> 6, col = r & 63, kg = col >> 3;
+    const int src = (kg < 4 ? 0 : PF_KHALF) + q * 32 + (kg & 3) * 8 + (col & 7);
+    img[(long)q * N * 64 + (row >> 3) * 512 + kg * 64 + (row & 7) * 8 + (col & 7)] =
+        B[(long)row * ldb + src];
+}
+
 __global__ void k_c128_to_c64(long n, const double2 *in, float2 *out) {
     const long i = (long)blockIdx.x * PTC_BLOCK + threadIdx.x;
     if (i < n) out[i] = make_float2((float)in[i].x, (float)in[i].y);
@@ -424,6 +439,7 @@ struct wd_ptc {
     float *F[PTC_MAX_LAYERS + 1] = {};        // activations, FP32
     __nv_bfloat16 *A[PTC_MAX_LAYERS] = {};    // gathered operands, BF16
     __nv_bfloat16 *B[PTC_MAX_LAYERS] = {};    // weight matrices, BF16
+    __nv_bfloat16 *Bimg[PTC_MAX_LAYERS] = {}; // the same as the fused layer's chunk images
     float2 *W[PTC_MAX_LAYERS] = {};           // complex weights (FP32 master copy)
     long wcount[PTC_MAX_LAYERS] = {};
     float2 *U = nullptr;                      // links, complex64 [V][4][3][3]
@@ -602,6 +618,11 @@ static int ptc_check_err(wd_ptc *n) {
     return WD_OK;
 }
 
+// whether layer l has a fused form: 16 input and 16 or 1 output channels
+static bool ptc_fusable(const wd_ptc *n, int l) {
+    return n->ch[l] == PF_CIN && (n->ch[l + 1] == 16 || n->ch[l + 1] == 1);
+}
+
 // One fused layer with 16 input channels (ptc_fused.cuh): F[l + 1] from
 // F[l], no gathered operand.
 template <int COUT>
@@ -613,6 +634,12 @@ static int ptc_layer_fused_t(wd_ptc *n, int l) {
         PTC_CUDA(cudaFuncSetAttribute(k_ptc_layer_fused<COUT>,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       pf_smem_bytes<COUT>()));
+        // the kernel's register hand-over needs this many at launch (with
+        // fewer it would wait for ever)
+        cudaFuncAttributes fa;
+        PTC_CUDA(cudaFuncGetAttributes(&fa, k_ptc_layer_fused<COUT>));
+        if (fa.numRegs * PF_ALL_THREADS < PF_REGS_TOTAL)
+            return ptc_fail(WD_ERR_CUDA, "fused layer built with too few registers per thread");
         if (dev >= 0 && dev < 64) attr_done[dev] = true;
     }
     if (n->Np[l] != pf_n<COUT>()) return ptc_fail(WD_ERR_ARG, "fused layer: output width");
@@ -621,10 +648,12 @@ static int ptc_layer_fused_t(wd_ptc *n, int l) {
     PfArgs a;
     a.g = n->g;
     a.F = n->F[l];
-    a.ldf = n->ldF[l];
+    if (n->ldF[l] != PF_LDF) return ptc_fail(WD_ERR_ARG, "fused layer: input width");
+    a.phase_on = 0;
+    for (int mu = 0; mu < 4; ++mu)
+        if (n->g.ph[2 * mu] != 1.0f || n->g.ph[2 * mu + 1] != 0.0f) a.phase_on |= 1u << mu;
     a.U = n->U;
-    a.B = n->B[l];
-    a.ldb = n->Kp[l];
+    a.B = n->Bimg[l];
     a.out = n->F[l + 1];
     a.ldo = n->ldF[l + 1];
     a.ntiles = (n->g.V + PF_SITES - 1) / PF_SITES;
@@ -652,8 +681,7 @@ static int ptc_forward(wd_ptc *n, const double *r, double in_scale, bool keep_op
     PTC_CUDA(cudaGetLastError());
     for (int l = 0; l < n->nl; ++l) {
         const int cin = n->ch[l];
-        if (!keep_operands && n->fused && cin == PF_CIN &&
-            (n->ch[l + 1] == 16 || n->ch[l + 1] == 1)) {
+        if (!keep_operands && n->fused && ptc_fusable(n, l)) {
             PTC_TRY(ptc_layer_fused(n, l));
             continue;
         }
@@ -724,6 +752,8 @@ int wd_ptc_create(wd_ptc **out, const int dims[4], const double phase[8], int nl
     for (int l = 0; l < nlayers && rc == WD_OK; ++l) {
         rc = ptc_alloc(n, (void **)&n->A[l], sizeof(__nv_bfloat16) * n->Mp * n->Kp[l]);
         if (rc == WD_OK) rc = ptc_alloc(n, (void **)&n->B[l], sizeof(__nv_bfloat16) * (long)n->Np[l] * n->Kp[l]);
+        if (rc == WD_OK && ptc_fusable(n, l))
+            rc = ptc_alloc(n, (void **)&n->Bimg[l], sizeof(__nv_bfloat16) * PF_NCHUNK * n->Np[l] * 64);
         if (rc == WD_OK) rc = ptc_alloc(n, (void **)&n->W[l], sizeof(float2) * n->wcount[l]);
     }
     if (rc == WD_OK) rc = ptc_alloc(n, (void **)&n->U, sizeof(float2) * V * 36);
@@ -751,6 +781,9 @@ static int ptc_rebuild_b(wd_ptc *n) {
         const long cnt = (long)n->ch[l + 1] * 4 * n->ch[l] * 36;
         k_ptc_weights<<<grid_for(cnt), PTC_BLOCK, 0, n->stream>>>(n->ch[l + 1], n->ch[l], n->W[l],
                                                                    n->B[l], n->Kp[l]);
+        if (n->Bimg[l])
+            k_ptc_weights_fused<<<grid_for((long)PF_NCHUNK * n->Np[l] * 64), PTC_BLOCK, 0,
+                                  n->stream>>>(n->Np[l], n->B[l], n->Kp[l], n->Bimg[l]);
         if (n->train_ready)
             k_ptc_weights_t<<<grid_for(cnt), PTC_BLOCK, 0, n->stream>>>(
                 n->ch[l + 1], n->ch[l], n->W[l], n->Bt[l], n->Rp[l + 1]);
