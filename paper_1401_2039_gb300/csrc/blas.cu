@@ -254,7 +254,7 @@ __global__ void k_f64_df64(long n, void *buf, int to_df) {
             reinterpret_cast<float2 *>(buf)[i] = make_float2(v.hi, v.lo);
         } else {
             const float2 f = reinterpret_cast<float2 *>(buf)[i];
-            reinterpret_cast<double *>(buf)[i] = (double)f.x + (double)f.y;
+            reinterpret_cast<double *>(buf)[i] = join_double(f.x, f.y);
         }
     }
 }

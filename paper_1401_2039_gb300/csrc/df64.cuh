@@ -25,35 +25,93 @@ struct __align__(8) df64 {
     __host__ __device__ constexpr df64(float h, float l) : hi(h), lo(l) {}
     __host__ __device__ constexpr df64(int v) : hi((float)v), lo(0.0f) {}
     __host__ __device__ df64(double d);
-    __host__ __device__ explicit operator double() const { return (double)hi + (double)lo; }
+    __host__ __device__ explicit operator double() const;
 };
 
 // hi = d rounded to FP32, lo = (d - hi) rounded to FP32.  On the device the
 // split is done on the bit pattern: GB300's FP64 adder runs at a small
 // fraction of the FP32 rate (a DADD per element made the canonical-to-
 // double-float conversion three times slower than a copy), while integer
-// operations and the narrowing conversion do not touch it.  Exact halfway
-// cases of hi round away from zero instead of to even.  Zeros, values below
-// 2^-74 or from 2^127 in magnitude, infinities and NaNs take the FP64 route.
+// operations do not touch it.  Exact halfway cases of hi round away from zero
+// instead of to even.  Nonzero values below 2^-74 or from 2^127 in magnitude,
+// infinities and NaNs take the FP64 route (zeros, most of a point source, must
+// not: they made the batched solver's packing of one 3.8 times slower).
 __device__ __forceinline__ df64 split_double(double d) {
     const unsigned long long u = (unsigned long long)__double_as_longlong(d);
     const int e = (int)((u >> 52) & 0x7FF) - 1023;
-    if (e < -74 || e > 126) {
-        if ((u << 1) == 0) return df64(__double2float_rn(d), 0.0f);   // +-0
+    const bool zero = (u << 1) == 0;
+    if ((e < -74 || e > 126) && !zero) {
         const float h = __double2float_rn(d);
         return df64(h, __double2float_rn(d - (double)h));
     }
     const unsigned long long m = u & 0xFFFFFFFFFFFFFull;
-    unsigned int hb = ((unsigned int)(u >> 32) & 0x80000000u) |
-                      ((unsigned int)(e + 127) << 23) | (unsigned int)(m >> 29);
+    const unsigned int sign = (unsigned int)(u >> 32) & 0x80000000u;
+    unsigned int hb = ((unsigned int)(e + 127) << 23) | (unsigned int)(m >> 29);
     int r = (int)(m & 0x1FFFFFFFu);          // the 29 bits below hi's last
     if (r >= (1 << 28)) {                    // round hi up, remainder negative
         hb += 1u;
         r -= (1 << 29);
     }
     float lo = __int2float_rn(r) * __int_as_float((e - 52 + 127) << 23);
-    if (u >> 63) lo = -lo;
-    return df64(__uint_as_float(hb), lo);
+    if (sign) lo = -lo;
+    return df64(__uint_as_float(sign | (zero ? 0u : hb)), zero ? 0.0f : lo);
+}
+
+// (double)hi + (double)lo, its bits exactly.  A normalised pair needs no FP64
+// addition: in units of the last place of the double that hi starts, lo is a
+// number of at most 29 bits, and rounding it to an integer (halfway to even,
+// as hi's own units are even) rounds the sum.  A lo that takes hi = +-2^e below
+// its binade counts in the half units of the lower one.  Other pairs take the
+// FP64 route (2 conversions and an addition per real, on the slow pipe).
+__device__ __forceinline__ double join_double(float hi, float lo) {
+    const unsigned int h = __float_as_uint(hi), l = __float_as_uint(lo);
+    const unsigned int m = h & 0x7FFFFFu, differ = (h ^ l) >> 31;
+    const int e = (int)((h >> 23) & 0xFF) - 127;
+    const int k = 52 - e + (m == 0 ? (int)differ : 0);
+    const float n = fabsf(lo) * __uint_as_float((unsigned int)(k + 127) << 23);
+    const bool zero = ((h | l) << 1) == 0;
+    if ((e < -74 || e > 127 || !(n <= 536870912.0f)) && !zero) return (double)hi + (double)lo;
+    const unsigned long long u =
+        (unsigned long long)((h & 0x80000000u) | (unsigned int)(e + 1023) << 20 | m >> 3) << 32 |
+        (unsigned long long)(m << 29);
+    const long long q = __float2int_rn(n);
+    const unsigned long long v = u + (unsigned long long)(differ ? -q : q);
+    return zero ? __hiloint2double((int)(h & l), 0) : __longlong_as_double((long long)v);
+}
+
+// FP64 -> FP32 (round to nearest even) and back for records that are
+// converted in bulk: the bits of the conversion instructions, which run on the
+// FP64 pipe (2 a clock and SM, the time of the layout kernels), from integer
+// ones.  Values that are not normal FP32 numbers or zeros leave them to the
+// instructions: *_ok tells.
+__device__ __forceinline__ bool narrow_ok(double d) {
+    const unsigned int h = (unsigned int)__double2hiint(d) & 0x7FFFFFFFu;
+    // [2^-126, 2^127), or zero
+    return h - 0x38100000u < 0x0FD00000u || (h | (unsigned int)__double2loint(d)) == 0;
+}
+__device__ __forceinline__ float narrow_double(double d) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(d);
+    const unsigned int h = (unsigned int)(u >> 32);
+    const unsigned long long t = u + 0x0FFFFFFFu + ((unsigned int)u >> 29 & 1u);
+    const unsigned int b = ((unsigned int)(t >> 29) - 0xC0000000u) & 0x7FFFFFFFu;
+    return __uint_as_float((h & 0x80000000u) | ((h << 1) == 0 ? 0u : b));
+}
+__device__ __forceinline__ bool widen_ok(float f) {
+    const unsigned int h = __float_as_uint(f) & 0x7FFFFFFFu;
+    return h - 0x00800000u < 0x7F000000u || h == 0;   // normal, or zero
+}
+__device__ __forceinline__ double widen_float(float f) {
+    const unsigned int h = __float_as_uint(f);
+    const unsigned int m = ((h & 0x7FFFFFFFu) >> 3) + (896u << 20);
+    return __hiloint2double((int)((h & 0x80000000u) | ((h << 1) == 0 ? 0u : m)), (int)(h << 29));
+}
+
+__host__ __device__ inline df64::operator double() const {
+#ifdef __CUDA_ARCH__
+    return join_double(hi, lo);
+#else
+    return (double)hi + (double)lo;
+#endif
 }
 
 __host__ __device__ inline df64::df64(double d) {

@@ -21,73 +21,114 @@ __device__ __forceinline__ void load_canonical(const double *src, long site, dou
     }
 }
 
-// Spinor records (24 doubles, 12 chunks of 16 bytes) of a block's
-// LAYOUT_BLOCK consecutive sites pass through shared memory: the canonical
-// side moves the block's contiguous chunks with consecutive threads on
-// consecutive chunks (coalesced), the internal side handles one record per
-// thread.  Records are padded to 13 chunks in shared memory, so that the
-// per-record accesses of 8 consecutive threads fall in distinct banks.
+// Spinor records (12 complex numbers) of a block's LAYOUT_BLOCK consecutive
+// sites pass through shared memory: the canonical side moves the block's
+// contiguous 16-byte chunks with consecutive threads on consecutive chunks
+// (coalesced), the internal side handles one record per thread.  A complex
+// number is held there in its storage precision, so that blocks of the 16-bit
+// types are bounded by threads and not by shared memory, and records are
+// padded to 13 numbers, so that the per-record accesses of consecutive threads
+// fall in distinct banks.  Memory bound, once the conversions leave the FP64
+// pipe and all of a thread's 12 loads are under way together.  BF16, one parity
+// of 28 x 20 x 36 x 46 (111 MB): in 26.6 -> 18.4 us, out 23.3 -> 15 us; the 16.3
+// us of a copy.  (Integer conversions alone left the way in at 26.0.)
 constexpr int SPIN_CHUNKS = 12, SPIN_PAD = 13;
 
+template <typename S> struct Staged {
+    static constexpr int WORDS = 2 * (int)sizeof(S) / 4;   // per complex number
+    using T = std::conditional_t<WORDS == 4, uint4, std::conditional_t<WORDS == 2, uint2, uint32_t>>;
+    __device__ __forceinline__ static T of(double2 d) {
+        const double v[2] = {d.x, d.y};
+        union { uint32_t w[WORDS]; T t; } u;
+        Words<S, double>::pack(v, u.w, 2);
+        return u.t;
+    }
+    __device__ __forceinline__ static double2 to(T t) {
+        union { uint32_t w[WORDS]; T t; } u;
+        u.t = t;
+        double v[2];
+        Words<S, double>::unpack(u.w, v, 2);
+        return make_double2(v[0], v[1]);
+    }
+};
+
+template <typename S>
 __device__ __forceinline__ void canonical_block_in(const double *src, long first, long n,
-                                                   double2 *sm) {
+                                                   typename Staged<S>::T *sm) {
     const double2 *g = reinterpret_cast<const double2 *>(src) + first * SPIN_CHUNKS;
     const long left = n - first;
     const int avail = (int)((left < LAYOUT_BLOCK ? left : LAYOUT_BLOCK) * SPIN_CHUNKS);
-#pragma unroll 4
-    for (int c = threadIdx.x; c < avail; c += LAYOUT_BLOCK)
-        sm[(c / SPIN_CHUNKS) * SPIN_PAD + c % SPIN_CHUNKS] = __ldcs(g + c);
+    double2 d[SPIN_CHUNKS];
+#pragma unroll
+    for (int k = 0; k < SPIN_CHUNKS; ++k) {
+        const int c = threadIdx.x + k * LAYOUT_BLOCK;
+        d[k] = c < avail ? __ldcs(g + c) : make_double2(0.0, 0.0);
+    }
+#pragma unroll
+    for (int k = 0; k < SPIN_CHUNKS; ++k) {
+        const int c = threadIdx.x + k * LAYOUT_BLOCK;
+        sm[(c / SPIN_CHUNKS) * SPIN_PAD + c % SPIN_CHUNKS] = Staged<S>::of(d[k]);
+    }
 }
 
+template <typename S>
 __device__ __forceinline__ void canonical_block_out(double *dst, long first, long n,
-                                                    const double2 *sm) {
+                                                    const typename Staged<S>::T *sm) {
     double2 *g = reinterpret_cast<double2 *>(dst) + first * SPIN_CHUNKS;
     const long left = n - first;
     const int avail = (int)((left < LAYOUT_BLOCK ? left : LAYOUT_BLOCK) * SPIN_CHUNKS);
 #pragma unroll 4
-    for (int c = threadIdx.x; c < avail; c += LAYOUT_BLOCK)
-        __stcs(g + c, sm[(c / SPIN_CHUNKS) * SPIN_PAD + c % SPIN_CHUNKS]);
-}
-
-__device__ __forceinline__ void record_from_smem(const double2 *sm, double *v) {
-    const double2 *p = sm + threadIdx.x * SPIN_PAD;
-#pragma unroll
-    for (int i = 0; i < SPIN_CHUNKS; ++i) {
-        const double2 d = p[i];
-        v[2 * i] = d.x;
-        v[2 * i + 1] = d.y;
+    for (int k = 0; k < SPIN_CHUNKS; ++k) {
+        const int c = threadIdx.x + k * LAYOUT_BLOCK;
+        if (c < avail)
+            __stcs(g + c, Staged<S>::to(sm[(c / SPIN_CHUNKS) * SPIN_PAD + c % SPIN_CHUNKS]));
     }
 }
 
-__device__ __forceinline__ void record_to_smem(double2 *sm, const double *v) {
-    double2 *p = sm + threadIdx.x * SPIN_PAD;
+// a thread's record between shared memory and the internal layout
+template <typename S>
+__device__ __forceinline__ void record_store(const typename Staged<S>::T *sm, void *dst,
+                                             long stride, long h) {
+    using St = Staged<S>;
+    union { uint32_t w[SPIN_CHUNKS * St::WORDS]; typename St::T t[SPIN_CHUNKS]; } u;
 #pragma unroll
-    for (int i = 0; i < SPIN_CHUNKS; ++i) p[i] = make_double2(v[2 * i], v[2 * i + 1]);
+    for (int i = 0; i < SPIN_CHUNKS; ++i) u.t[i] = sm[threadIdx.x * SPIN_PAD + i];
+#pragma unroll
+    for (int j = 0; j < Rec<S, 24>::NF; ++j)
+        st_v4((char *)dst + ((long)j * stride + h) * 16,
+              make_uint4(u.w[4 * j], u.w[4 * j + 1], u.w[4 * j + 2], u.w[4 * j + 3]));
+}
+
+template <typename S>
+__device__ __forceinline__ void record_load(typename Staged<S>::T *sm, const void *src,
+                                            long stride, long h) {
+    using St = Staged<S>;
+    union { uint32_t w[SPIN_CHUNKS * St::WORDS]; typename St::T t[SPIN_CHUNKS]; } u;
+#pragma unroll
+    for (int j = 0; j < Rec<S, 24>::NF; ++j) {
+        const uint4 v = ld_v4((const char *)src + ((long)j * stride + h) * 16);
+        u.w[4 * j] = v.x; u.w[4 * j + 1] = v.y; u.w[4 * j + 2] = v.z; u.w[4 * j + 3] = v.w;
+    }
+#pragma unroll
+    for (int i = 0; i < SPIN_CHUNKS; ++i) sm[threadIdx.x * SPIN_PAD + i] = u.t[i];
 }
 
 template <typename S>
 __global__ void __launch_bounds__(LAYOUT_BLOCK) k_pack_half(Geom g, void *dst, const double *src) {
-    __shared__ double2 sm[LAYOUT_BLOCK * SPIN_PAD];
+    __shared__ typename Staged<S>::T sm[LAYOUT_BLOCK * SPIN_PAD];
     const long first = (long)blockIdx.x * LAYOUT_BLOCK, h = first + threadIdx.x;
-    canonical_block_in(src, first, g.vh, sm);
+    canonical_block_in<S>(src, first, g.vh, sm);
     __syncthreads();
-    if (h >= g.vh) return;
-    double v[24];
-    record_from_smem(sm, v);
-    Rec<S, 24>::store(dst, g.stride, h, v);
+    if (h < g.vh) record_store<S>(sm, dst, g.stride, h);
 }
 
 template <typename S>
 __global__ void __launch_bounds__(LAYOUT_BLOCK) k_unpack_half(Geom g, double *dst, const void *src) {
-    __shared__ double2 sm[LAYOUT_BLOCK * SPIN_PAD];
+    __shared__ typename Staged<S>::T sm[LAYOUT_BLOCK * SPIN_PAD];
     const long first = (long)blockIdx.x * LAYOUT_BLOCK, h = first + threadIdx.x;
-    if (h < g.vh) {
-        double v[24];
-        Rec<S, 24>::template load_coherent<double>(src, g.stride, h, v);
-        record_to_smem(sm, v);
-    }
+    if (h < g.vh) record_load<S>(sm, src, g.stride, h);
     __syncthreads();
-    canonical_block_out(dst, first, g.vh, sm);
+    canonical_block_out<S>(dst, first, g.vh, sm);
 }
 
 // parity of lexicographic site lex (32-bit arithmetic: volumes stay below 2^31;
@@ -108,29 +149,22 @@ template <typename S>
 __global__ void __launch_bounds__(LAYOUT_BLOCK) k_pack_full(Geom g, void *even, void *odd,
                                                             const double *src, long lex0,
                                                             long lex1) {
-    __shared__ double2 sm[LAYOUT_BLOCK * SPIN_PAD];
+    __shared__ typename Staged<S>::T sm[LAYOUT_BLOCK * SPIN_PAD];
     const long first = lex0 + (long)blockIdx.x * LAYOUT_BLOCK, lex = first + threadIdx.x;
-    canonical_block_in(src, first, lex1, sm);
+    canonical_block_in<S>(src, first, lex1, sm);
     __syncthreads();
-    if (lex >= lex1) return;
-    double v[24];
-    record_from_smem(sm, v);
-    Rec<S, 24>::store(lex_parity(g, lex) ? odd : even, g.stride, lex >> 1, v);
+    if (lex < lex1) record_store<S>(sm, lex_parity(g, lex) ? odd : even, g.stride, lex >> 1);
 }
 
 template <typename S>
 __global__ void __launch_bounds__(LAYOUT_BLOCK) k_unpack_full(Geom g, double *dst, const void *even,
                                                               const void *odd) {
-    __shared__ double2 sm[LAYOUT_BLOCK * SPIN_PAD];
+    __shared__ typename Staged<S>::T sm[LAYOUT_BLOCK * SPIN_PAD];
     const long first = (long)blockIdx.x * LAYOUT_BLOCK, lex = first + threadIdx.x;
-    if (lex < 2 * g.vh) {
-        double v[24];
-        Rec<S, 24>::template load_coherent<double>(lex_parity(g, lex) ? odd : even, g.stride,
-                                                    lex >> 1, v);
-        record_to_smem(sm, v);
-    }
+    if (lex < 2 * g.vh)
+        record_load<S>(sm, lex_parity(g, lex) ? odd : even, g.stride, lex >> 1);
     __syncthreads();
-    canonical_block_out(dst, first, 2 * g.vh, sm);
+    canonical_block_out<S>(dst, first, 2 * g.vh, sm);
 }
 
 // One thread per (site, direction): the link's first RECON reals (row-major,

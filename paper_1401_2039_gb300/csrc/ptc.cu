@@ -43,20 +43,31 @@ __global__ void k_ptc_in(long V, const double2 *__restrict__ r, float *__restric
     const long i = (long)blockIdx.x * PTC_BLOCK + threadIdx.x;   // (x, a)
     if (i >= 3 * V) return;
     float *row = F + i * ld;
+    double v[8];
+    uint32_t w[8];
+#pragma unroll
     for (int s = 0; s < 4; ++s) {
-        const double2 v = r[i * 4 + s];
-        row[s] = (float)v.x * scale;
-        row[4 + s] = (float)v.y * scale;
+        const double2 c = r[i * 4 + s];
+        v[s] = c.x;
+        v[4 + s] = c.y;
     }
+    Words<float, double>::pack(v, w, 8);
+#pragma unroll
+    for (int s = 0; s < 8; ++s) row[s] = __uint_as_float(w[s]) * scale;
 }
 
-// F rows (x, a) [Re s0..3, Im s0..3] -> canonical complex128, times scale
-__global__ void k_ptc_out(long V, const float *__restrict__ F, int ld, double2 *__restrict__ y,
-                          double scale) {
+// F rows (x, a) [Re s0..3, Im s0..3] -> canonical complex128
+__global__ void k_ptc_out(long V, const float *__restrict__ F, int ld, double2 *__restrict__ y) {
     const long i = (long)blockIdx.x * PTC_BLOCK + threadIdx.x;
     if (i >= 3 * V) return;
     const float *row = F + i * ld;
-    for (int s = 0; s < 4; ++s) y[i * 4 + s] = make_double2(row[s] * scale, row[4 + s] * scale);
+    double v[8];
+    uint32_t w[8];
+#pragma unroll
+    for (int s = 0; s < 8; ++s) w[s] = __float_as_uint(row[s]);
+    Words<float, double>::unpack(w, v, 8);
+#pragma unroll
+    for (int s = 0; s < 4; ++s) y[i * 4 + s] = make_double2(v[s], v[4 + s]);
 }
 
 struct PtcGeom {
@@ -938,7 +949,7 @@ int wd_ptc_apply(wd_ptc *n, double *y, const double *r) {
     PTC_TRY(ptc_fork(n));
     PTC_TRY(ptc_forward(n, r, 1.0));
     k_ptc_out<<<grid_for(3 * n->g.V), PTC_BLOCK, 0, n->stream>>>(
-        n->g.V, n->F[n->nl], n->ldF[n->nl], (double2 *)y, 1.0);
+        n->g.V, n->F[n->nl], n->ldF[n->nl], (double2 *)y);
     PTC_CUDA(cudaGetLastError());
     PTC_TRY(ptc_check_err(n));
     return ptc_join(n);

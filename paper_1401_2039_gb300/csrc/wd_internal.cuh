@@ -152,13 +152,29 @@ template <typename S> struct WordsViaFloat {
     __device__ static void unpack(const uint32_t *w, double *r, int n) {
         float f[24];
         Words<S, float>::unpack(w, f, n);
+        bool ok = true;
 #pragma unroll
-        for (int i = 0; i < n; ++i) r[i] = (double)f[i];
+        for (int i = 0; i < n; ++i) ok &= widen_ok(f[i]);
+        if (ok) {
+#pragma unroll
+            for (int i = 0; i < n; ++i) r[i] = widen_float(f[i]);
+        } else {
+#pragma unroll
+            for (int i = 0; i < n; ++i) r[i] = (double)f[i];
+        }
     }
     __device__ static void pack(const double *r, uint32_t *w, int n) {
         float f[24];
+        bool ok = true;
 #pragma unroll
-        for (int i = 0; i < n; ++i) f[i] = (float)r[i];
+        for (int i = 0; i < n; ++i) ok &= narrow_ok(r[i]);
+        if (ok) {
+#pragma unroll
+            for (int i = 0; i < n; ++i) f[i] = narrow_double(r[i]);
+        } else {
+#pragma unroll
+            for (int i = 0; i < n; ++i) f[i] = (float)r[i];
+        }
         Words<S, float>::pack(f, w, n);
     }
 };
@@ -185,7 +201,7 @@ template <> struct Words<df64, double> {
     __device__ static void unpack(const uint32_t *w, double *r, int n) {
 #pragma unroll
         for (int i = 0; i < n; ++i)
-            r[i] = (double)__uint_as_float(w[2 * i]) + (double)__uint_as_float(w[2 * i + 1]);
+            r[i] = join_double(__uint_as_float(w[2 * i]), __uint_as_float(w[2 * i + 1]));
     }
     __device__ static void pack(const double *r, uint32_t *w, int n) {
 #pragma unroll
