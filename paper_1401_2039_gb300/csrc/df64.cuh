@@ -28,6 +28,21 @@ struct __align__(8) df64 {
     __host__ __device__ explicit operator double() const;
 };
 
+// The conversion instructions, for values that the integer forms below leave
+// to them.  Called, not inlined: a short FP64 block behind a condition is
+// turned into predicated instructions, and those occupy the slow FP64 pipe
+// whether or not any lane needs them (2.1 ms instead of 0.8 for packing the
+// batched solver's right-hand sides).
+static __device__ __noinline__ float narrow_slow(double d) { return __double2float_rn(d); }
+static __device__ __noinline__ double widen_slow(float f) { return (double)f; }
+static __device__ __noinline__ float2 split_slow(double d) {
+    const float h = __double2float_rn(d);
+    return make_float2(h, __double2float_rn(d - (double)h));
+}
+static __device__ __noinline__ double join_slow(float hi, float lo) {
+    return (double)hi + (double)lo;
+}
+
 // hi = d rounded to FP32, lo = (d - hi) rounded to FP32.  On the device the
 // split is done on the bit pattern: GB300's FP64 adder runs at a small
 // fraction of the FP32 rate (a DADD per element made the canonical-to-
@@ -39,10 +54,11 @@ struct __align__(8) df64 {
 __device__ __forceinline__ df64 split_double(double d) {
     const unsigned long long u = (unsigned long long)__double_as_longlong(d);
     const int e = (int)((u >> 52) & 0x7FF) - 1023;
-    const bool zero = (u << 1) == 0;
+    // (of the halves: a test of the whole pattern is compiled to an FP64 compare)
+    const bool zero = (((unsigned int)(u >> 32) << 1) | (unsigned int)u) == 0;
     if ((e < -74 || e > 126) && !zero) {
-        const float h = __double2float_rn(d);
-        return df64(h, __double2float_rn(d - (double)h));
+        const float2 v = split_slow(d);
+        return df64(v.x, v.y);
     }
     const unsigned long long m = u & 0xFFFFFFFFFFFFFull;
     const unsigned int sign = (unsigned int)(u >> 32) & 0x80000000u;
@@ -70,7 +86,7 @@ __device__ __forceinline__ double join_double(float hi, float lo) {
     const int k = 52 - e + (m == 0 ? (int)differ : 0);
     const float n = fabsf(lo) * __uint_as_float((unsigned int)(k + 127) << 23);
     const bool zero = ((h | l) << 1) == 0;
-    if ((e < -74 || e > 127 || !(n <= 536870912.0f)) && !zero) return (double)hi + (double)lo;
+    if ((e < -74 || e > 127 || !(n <= 536870912.0f)) && !zero) return join_slow(hi, lo);
     const unsigned long long u =
         (unsigned long long)((h & 0x80000000u) | (unsigned int)(e + 1023) << 20 | m >> 3) << 32 |
         (unsigned long long)(m << 29);

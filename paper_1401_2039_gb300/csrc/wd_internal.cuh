@@ -160,7 +160,7 @@ template <typename S> struct WordsViaFloat {
             for (int i = 0; i < n; ++i) r[i] = widen_float(f[i]);
         } else {
 #pragma unroll
-            for (int i = 0; i < n; ++i) r[i] = (double)f[i];
+            for (int i = 0; i < n; ++i) r[i] = widen_slow(f[i]);
         }
     }
     __device__ static void pack(const double *r, uint32_t *w, int n) {
@@ -173,7 +173,7 @@ template <typename S> struct WordsViaFloat {
             for (int i = 0; i < n; ++i) f[i] = narrow_double(r[i]);
         } else {
 #pragma unroll
-            for (int i = 0; i < n; ++i) f[i] = (float)r[i];
+            for (int i = 0; i < n; ++i) f[i] = narrow_slow(r[i]);
         }
         Words<S, float>::pack(f, w, n);
     }
