@@ -47,18 +47,19 @@ template <> __device__ __forceinline__ df64 bt_fma<df64>(df64 a, df64 b, df64 c)
 template <typename S, typename R, int OP>
 __global__ void __launch_bounds__(BT_BLOCK) k_bt_vec(const __grid_constant__ BtArgs a) {
     using C = Chunk16<S, R>;
-    __shared__ df64 wv[BT_BLOCK];
+    __shared__ df64 wv[BT_WARPS][BT_DEFER][32];
     __shared__ df64 wacc[BT_WARPS][BT_MAX_SLOTS];
     __shared__ df64 sacc[BT_MAX_SLOTS];
     constexpr bool RED = OP == BT_R || OP == BT_NORM;
     if (RED) bt_zero_sums(wacc);
+    BtDeferred kept;
     for (long t = blockIdx.x; t < a.ntiles; t += gridDim.x) {
-        const BtProb &P = a.p[bt_problem(a, t)];
-        const long item0 = (t - P.tile0) * BT_BLOCK;
-        const long i = item0 + threadIdx.x;
+        const int prob = bt_problem(a, t);
+        const BtProb &P = a.p[prob];
+        const long i = (t - P.tile0) * BT_BLOCK + threadIdx.x;
         df64 v = 0;
         if (i < P.nitems) {
-            SolverScalars *s = &a.scalars[P.slot0 + (int)((unsigned)i % (unsigned)P.nrhs)];
+            SolverScalars *s = &a.scalars[P.slot0 + bt_rhs(P, i)];
             if (OP == BT_R) {           // f = {r, Ap}: r -= a Ap, |r|^2
                 const R al = (R)s->alpha;
                 R rv[C::K], av[C::K];
@@ -93,7 +94,7 @@ __global__ void __launch_bounds__(BT_BLOCK) k_bt_vec(const __grid_constant__ BtA
                 for (int k = 0; k < C::K; ++k) sq += vv[k] * vv[k];
                 v = to_df(sq);
             } else {                    // f = {p}: p *= ratio[slot]
-                const int slot = P.slot0 + (int)((unsigned)i % (unsigned)P.nrhs);
+                const int slot = P.slot0 + bt_rhs(P, i);
                 const R ratio = (R)a.consts[2 * BT_MAX_SLOTS + slot];
                 R pv[C::K];
                 C::load(P.f[0], i, pv);
@@ -102,9 +103,10 @@ __global__ void __launch_bounds__(BT_BLOCK) k_bt_vec(const __grid_constant__ BtA
                 C::store(P.f[0], i, pv);
             }
         }
-        if (RED) bt_warp_sums(v, P, item0, wv, wacc);
+        if (RED) bt_defer(a, kept, prob, t, v, wv, wacc);
     }
     if (RED) {
+        bt_flush(a, kept, wv, wacc);
         bt_block_sums(wacc, sacc, a.nslots);
         bt_finish(a, sacc);
     }
@@ -118,14 +120,15 @@ enum BtOp64 { BT64_XMY = 0, BT64_XPAY = 1 };
 template <typename H, int OP>
 __global__ void __launch_bounds__(BT_BLOCK) k_bt_hi(const __grid_constant__ BtArgs a) {
     using C = Chunk16<H, H>;
-    __shared__ df64 wv[BT_BLOCK];
+    __shared__ df64 wv[BT_WARPS][BT_DEFER][32];
     __shared__ df64 wacc[BT_WARPS][BT_MAX_SLOTS];
     __shared__ df64 sacc[BT_MAX_SLOTS];
     if (OP == BT64_XMY) bt_zero_sums(wacc);
+    BtDeferred kept;
     for (long t = blockIdx.x; t < a.ntiles; t += gridDim.x) {
-        const BtProb &P = a.p[bt_problem(a, t)];
-        const long item0 = (t - P.tile0) * BT_BLOCK;
-        const long i = item0 + threadIdx.x;
+        const int prob = bt_problem(a, t);
+        const BtProb &P = a.p[prob];
+        const long i = (t - P.tile0) * BT_BLOCK + threadIdx.x;
         df64 v = 0;
         if (i < P.nitems) {
             H xv[C::K], yv[C::K], d[C::K];
@@ -141,9 +144,10 @@ __global__ void __launch_bounds__(BT_BLOCK) k_bt_hi(const __grid_constant__ BtAr
             C::store(P.f[0], i, d);
             v = to_df(sq);
         }
-        if (OP == BT64_XMY) bt_warp_sums(v, P, item0, wv, wacc);
+        if (OP == BT64_XMY) bt_defer(a, kept, prob, t, v, wv, wacc);
     }
     if (OP == BT64_XMY) {
+        bt_flush(a, kept, wv, wacc);
         bt_block_sums(wacc, sacc, a.nslots);
         bt_finish(a, sacc);
     }
@@ -207,59 +211,92 @@ __global__ void k_bt_rescale_nz(SolverScalars *sc, const double *consts, int nsl
     }
 }
 
-// item i of an [nrhs][V] enumeration: rhs r, lexicographic site lex and the
-// site's parity.  32-bit arithmetic (volumes stay below 2^31) except for the
-// rhs division of items past 2^32.
-__device__ __forceinline__ void bt_item_site(const Geom &g, long i, long V, int &r, long &lex,
-                                             int &par) {
-    if (i < (1L << 32)) {
-        const unsigned iu = (unsigned)i, Vu = (unsigned)V;
-        r = (int)(iu / Vu);
-        lex = (long)(iu - (unsigned)r * Vu);
+// One 16-byte chunk (two reals) of a field in the residual precision H <-> the
+// canonical pair of doubles.
+template <typename H> __device__ __forceinline__ uint4 bt_chunk_of(double2 d) {
+    const double v[2] = {d.x, d.y};
+    uint32_t w[4];
+    Words<H, double>::pack(v, w, 2);
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+template <typename H> __device__ __forceinline__ double2 bt_double_of(uint4 c) {
+    const uint32_t w[4] = {c.x, c.y, c.z, c.w};
+    double v[2];
+    Words<H, double>::unpack(w, v, 2);
+    return make_double2(v[0], v[1]);
+}
+
+// Canonical [nrhs][V][3][4] complex128 <-> batched parity fields (rhs index
+// innermost).  A block takes BTP_LEX consecutive sites (as many of either
+// parity) of BTP_RHS right-hand sides through shared memory: the canonical side
+// moves contiguous 16-byte chunks of each right-hand side, the field side runs
+// of (sites of a parity x right-hand sides) chunks per plane; chunk j of a
+// record is plane j, so the conversion is chunk by chunk.  Memory bound; with a
+// thread per record, 192 bytes apart on one side and nrhs chunks on the other,
+// 12 right-hand sides on 24^3 x 48 (3.06 GB) took 2.93 ms packed and 1.90 ms
+// unpacked; now 0.61 and 0.66 ms.
+// The pitches keep 8 consecutive chunks of either side in distinct banks.
+constexpr int BTP_LEX = 16, BTP_RHS = 12, BTP_BLOCK = 256;
+constexpr int BTP_SITE = 13, BTP_PITCH = BTP_LEX * BTP_SITE + 1;
+
+// parity of canonical site lex (32-bit: volumes stay below 2^31)
+__device__ __forceinline__ int bt_lex_parity(const Geom &g, unsigned lex) {
+    unsigned q = lex / (unsigned)g.L[0];
+    int par = (int)(lex - q * (unsigned)g.L[0]);
+    unsigned s = q / (unsigned)g.L[1];
+    par += (int)(q - s * (unsigned)g.L[1]);
+    q = s / (unsigned)g.L[2];
+    return (par + (int)(s - q * (unsigned)g.L[2]) + (int)q) & 1;
+}
+
+template <typename H, int UNPACK>
+__global__ void __launch_bounds__(BTP_BLOCK)
+k_bt_full(Geom g, int nrhs, Divisor div_full, Divisor div_last, void *even, void *odd,
+          double *canon) {
+    __shared__ uint4 sm[BTP_RHS * BTP_PITCH];
+    __shared__ int first[BTP_LEX / 2];   // parity of site 2 i of the block
+    const long lex0 = (long)blockIdx.x * BTP_LEX;
+    const int n = (int)min((long)BTP_LEX, 2 * g.vh - lex0);   // (even: Lx is)
+    const int r0 = blockIdx.y * BTP_RHS, R = min(BTP_RHS, nrhs - r0);
+    const Divisor divR = blockIdx.y + 1 == gridDim.y ? div_last : div_full;   // by R
+    if (threadIdx.x < n / 2)
+        first[threadIdx.x] = bt_lex_parity(g, (unsigned)(lex0 + 2 * threadIdx.x));
+    double2 *c2 = reinterpret_cast<double2 *>(canon) + ((long)r0 * 2 * g.vh + lex0) * 12;
+    const long rstep = 2 * g.vh * 12, plane = g.stride * nrhs;
+    constexpr int PER = BTP_LEX * 12;   // chunks of one right-hand side (a short block skips some)
+    auto canonical = [&](auto move) {
+#pragma unroll 3
+        for (int c = threadIdx.x; c < R * PER; c += BTP_BLOCK) {
+            const int r = c / PER, k = c - r * PER, s = k / 12;
+            if (s < n) move(c2 + r * rstep + k, r * BTP_PITCH + s * BTP_SITE + k - 12 * s);
+        }
+    };
+    // chunk c: right-hand side r innermost, then the pair of sites i, the parity, the plane
+    auto field = [&](auto move) {
+#pragma unroll 3
+        for (int c = threadIdx.x; c < R * PER; c += BTP_BLOCK) {
+            const int q = (int)udiv((unsigned)c, divR), r = c - q * R;
+            const int i = q & (BTP_LEX / 2 - 1), par = (q >> 3) & 1, j = q >> 4;
+            if (2 * i < n) {
+                const int s = 2 * i + (first[i] == par ? 0 : 1);
+                const long at = j * plane + ((lex0 >> 1) + i) * nrhs + r0 + r;
+                move(reinterpret_cast<uint4 *>(par ? odd : even) + at,
+                     r * BTP_PITCH + s * BTP_SITE + j);
+            }
+        }
+    };
+    if (UNPACK) {
+        __syncthreads();   // first[]
+        field([&](uint4 *p, int q) { sm[q] = *p; });
+        __syncthreads();
+        canonical([&](double2 *p, int q) { __stcs(p, bt_double_of<H>(sm[q])); });
     } else {
-        r = (int)(i / V);
-        lex = i - (long)r * V;
+        canonical([&](double2 *p, int q) { sm[q] = bt_chunk_of<H>(__ldcs(p)); });
+        __syncthreads();
+        field([&](uint4 *p, int q) { *p = sm[q]; });
     }
-    unsigned q = (unsigned)lex;
-    unsigned s = q / (unsigned)g.L[0];
-    par = (int)(q - s * (unsigned)g.L[0]);
-    q = s / (unsigned)g.L[1];
-    par += (int)(s - q * (unsigned)g.L[1]);
-    s = q / (unsigned)g.L[2];
-    par += (int)(q - s * (unsigned)g.L[2]) + (int)s;
-    par &= 1;
 }
-
-// Canonical [nrhs][V][3][4] complex128 <-> batched FP64 parity fields.
-template <typename H>
-__global__ void k_bt_pack_full(Geom g, int nrhs, void *even, void *odd, const double *src) {
-    const long i = (long)blockIdx.x * BT_BLOCK + threadIdx.x;
-    const long V = 2 * g.vh;
-    if (i >= V * nrhs) return;
-    int r, par;
-    long lex;
-    bt_item_site(g, i, V, r, lex, par);
-    double v[24];
-    const double2 *s2 = (const double2 *)(src + i * 24);
-    for (int k = 0; k < 12; ++k) { v[2 * k] = s2[k].x; v[2 * k + 1] = s2[k].y; }
-    Rec<H, 24>::store(par ? odd : even, g.stride * nrhs, (lex >> 1) * nrhs + r, v);
-}
-
-template <typename H>
-__global__ void k_bt_unpack_full(Geom g, int nrhs, double *dst, const void *even,
-                                 const void *odd) {
-    const long i = (long)blockIdx.x * BT_BLOCK + threadIdx.x;
-    const long V = 2 * g.vh;
-    if (i >= V * nrhs) return;
-    int r, par;
-    long lex;
-    bt_item_site(g, i, V, r, lex, par);
-    double v[24];
-    Rec<H, 24>::template load_coherent<double>(par ? odd : even, g.stride * nrhs,
-                                               (lex >> 1) * nrhs + r, v);
-    double2 *d2 = (double2 *)(dst + i * 24);
-    for (int k = 0; k < 12; ++k) d2[k] = make_double2(v[2 * k], v[2 * k + 1]);
-}
+static_assert(BTP_LEX == 16, "chunk indices of k_bt_full");
 
 // Canonical half spinors [nrhs][Vh][3][4] <-> a batched field of precision S.
 template <typename S, int UNPACK>
@@ -588,6 +625,24 @@ int bt_true_residual(wd_batch *bt, int p) {
     return WD_OK;
 }
 
+// canonical [nrhs][V] spinors -> the parity fields of problem p in the residual
+// precision (unpack: back)
+void bt_pack_full(wd_batch *bt, int p, void *even, void *odd, double *canon, int unpack) {
+    const wd_op *op = bt->ops[p];
+    const int nr = bt->nrhs[p];
+    const dim3 grid((unsigned)((2 * op->g.vh + BTP_LEX - 1) / BTP_LEX),
+                    (unsigned)((nr + BTP_RHS - 1) / BTP_RHS));
+    const Divisor df = make_divisor(BTP_RHS), dl = make_divisor((unsigned)((nr - 1) % BTP_RHS + 1));
+    cudaStream_t st = bt->stream;
+    if (bt->hi_prec == WD_DF64) {
+        if (unpack) k_bt_full<df64, 1><<<grid, BTP_BLOCK, 0, st>>>(op->g, nr, df, dl, even, odd, canon);
+        else k_bt_full<df64, 0><<<grid, BTP_BLOCK, 0, st>>>(op->g, nr, df, dl, even, odd, canon);
+    } else {
+        if (unpack) k_bt_full<double, 1><<<grid, BTP_BLOCK, 0, st>>>(op->g, nr, df, dl, even, odd, canon);
+        else k_bt_full<double, 0><<<grid, BTP_BLOCK, 0, st>>>(op->g, nr, df, dl, even, odd, canon);
+    }
+}
+
 int bt_solve_impl(wd_batch *bt, double *const *x, const double *const *b, double tol,
                   int maxiter, int par, wd_solve_info *info) {
     const int q = 1 - par;
@@ -599,20 +654,9 @@ int bt_solve_impl(wd_batch *bt, double *const *x, const double *const *b, double
     cudaStream_t st = bt->stream;
     // split b and x0 by parity into the FP64 batched fields
     for (int p = 0; p < bt->nprob; ++p) {
-        const wd_op *op = bt->ops[p];
-        const long n = 2 * op->g.vh * bt->nrhs[p];
-        const unsigned gr = (unsigned)((n + BT_BLOCK - 1) / BT_BLOCK);
-        double *xe = (double *)bt->fl[p].f[par == 0 ? F_XH : F_XQ];
-        double *xo = (double *)bt->fl[p].f[par == 0 ? F_XQ : F_XH];
-        if (bt->hi_prec == WD_DF64) {
-            k_bt_pack_full<df64><<<gr, BT_BLOCK, 0, st>>>(op->g, bt->nrhs[p], bt->fl[p].f[F_HB0],
-                                                          bt->fl[p].f[F_HB1], b[p]);
-            k_bt_pack_full<df64><<<gr, BT_BLOCK, 0, st>>>(op->g, bt->nrhs[p], xe, xo, x[p]);
-        } else {
-            k_bt_pack_full<double><<<gr, BT_BLOCK, 0, st>>>(op->g, bt->nrhs[p], bt->fl[p].f[F_HB0],
-                                                            bt->fl[p].f[F_HB1], b[p]);
-            k_bt_pack_full<double><<<gr, BT_BLOCK, 0, st>>>(op->g, bt->nrhs[p], xe, xo, x[p]);
-        }
+        void *xe = bt->fl[p].f[par == 0 ? F_XH : F_XQ], *xo = bt->fl[p].f[par == 0 ? F_XQ : F_XH];
+        bt_pack_full(bt, p, bt->fl[p].f[F_HB0], bt->fl[p].f[F_HB1], const_cast<double *>(b[p]), 0);
+        bt_pack_full(bt, p, xe, xo, x[p], 0);
     }
     BT_CUDA(cudaGetLastError());
     const int HBP = par == 0 ? F_HB0 : F_HB1, HBQ = par == 0 ? F_HB1 : F_HB0;
@@ -761,18 +805,14 @@ int bt_solve_impl(wd_batch *bt, double *const *x, const double *const *b, double
     else BT_TRY(bt_hop(bt, true, q, 0, F_XQ, F_XH, HBQ, SC_KAPPA, FIN_NONE));
     BT_TRY(bt_hop(bt, true, par, 0, F_AXH, F_XQ, F_XH, SC_MKAPPA, FIN_NONE));
     BT_TRY(bt_f64<BT64_XMY>(bt, FIN_STORE0, {F_RH, HBP, F_AXH}, SC_ONE));
-    BT_TRY(bt_hop(bt, true, q, 0, F_AXH, F_XH, F_XQ, SC_MKAPPA, FIN_NONE));
+    // x_q - kappa H_qp x_p from the last refresh's first hop, as in the
+    // single-system solver (x_p has not changed since)
+    if (th_valid) BT_TRY(bt_f64<BT64_XPAY>(bt, FIN_NONE, {F_AXH, F_XQ, F_TH}, SC_MKAPPA));
+    else BT_TRY(bt_hop(bt, true, q, 0, F_AXH, F_XH, F_XQ, SC_MKAPPA, FIN_NONE));
     BT_TRY(bt_f64<BT64_XMY>(bt, FIN_STORE1, {F_TH, HBQ, F_AXH}, SC_ONE));
     for (int p = 0; p < bt->nprob; ++p) {
-        const wd_op *op = bt->ops[p];
-        const long n = 2 * op->g.vh * bt->nrhs[p];
-        const unsigned gr = (unsigned)((n + BT_BLOCK - 1) / BT_BLOCK);
-        const double *xe = (const double *)bt->fl[p].f[par == 0 ? F_XH : F_XQ];
-        const double *xo = (const double *)bt->fl[p].f[par == 0 ? F_XQ : F_XH];
-        if (bt->hi_prec == WD_DF64)
-            k_bt_unpack_full<df64><<<gr, BT_BLOCK, 0, st>>>(op->g, bt->nrhs[p], x[p], xe, xo);
-        else
-            k_bt_unpack_full<double><<<gr, BT_BLOCK, 0, st>>>(op->g, bt->nrhs[p], x[p], xe, xo);
+        bt_pack_full(bt, p, bt->fl[p].f[par == 0 ? F_XH : F_XQ], bt->fl[p].f[par == 0 ? F_XQ : F_XH],
+                     x[p], 1);
     }
     BT_CUDA(cudaGetLastError());
     BT_TRY(bt_read(bt));

@@ -55,6 +55,15 @@ __device__ __forceinline__ int bt_problem(const BtArgs &a, long t) {
     return pi;
 }
 
+// right-hand side of item i of problem P, i % nrhs
+__device__ __forceinline__ int bt_rhs(const BtProb &P, long i) {
+    if (i < (1L << 31)) {
+        const unsigned u = (unsigned)i;
+        return (int)(u - udiv(u, P.div_nrhs) * (unsigned)P.nrhs);
+    }
+    return (int)(i % P.nrhs);
+}
+
 // Per-rhs sums of the items of a tile, without block barriers.  Each warp
 // stages its 32 values (items item0 + 32 w + lane; the item's rhs is item %
 // nrhs) in its own shared-memory row; lane j then adds the values of rhs j in
@@ -69,14 +78,77 @@ __device__ __forceinline__ void bt_warp_sums(df64 v, const BtProb &P, long item0
     wv[threadIdx.x] = v;
     __syncwarp();
     const int nr = P.nrhs;
-    const long iw = item0 + 32 * w;
-    const int base = (int)(iw % nr);
+    const int base = bt_rhs(P, item0 + 32 * w);
     for (int j = lane; j < nr; j += 32) {
         df64 s = 0;
-        for (int l = (j - base + nr) % nr; l < 32; l += nr) s = s + wv[32 * w + l];
+        for (int l = j < base ? j - base + nr : j - base; l < 32; l += nr) s = s + wv[32 * w + l];
         wacc[w][P.slot0 + j] = wacc[w][P.slot0 + j] + s;
     }
     __syncwarp();
+}
+
+// The same sums for the element-wise kernels, whose tiles are many and small:
+// a warp keeps the values of up to BT_DEFER of its tiles and then adds 32 /
+// nrhs tiles' right-hand sides side by side, one lane each, before it
+// accumulates them in tile order.  Every sum is the one bt_warp_sums forms, in
+// its order; with four right-hand sides a tile's eight dependent additions per
+// lane, on four lanes, took 14 of the update's 44 us on 176,640 sites.
+constexpr int BT_DEFER = 8;
+struct BtDeferred {
+    long t0 = 0;      // first tile kept (the others follow gridDim.x apart)
+    int n = 0;        // tiles kept
+    int prob = -1;    // their problem
+};
+__device__ __forceinline__ void bt_flush(const BtArgs &a, BtDeferred &d,
+                                         df64 (*wv)[BT_DEFER][32],
+                                         df64 (*wacc)[BT_MAX_SLOTS]) {
+    if (d.n == 0) return;
+    const BtProb &P = a.p[d.prob];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nr = P.nrhs;
+    __syncwarp();
+    if (nr > 32) {
+        for (int k = 0; k < d.n; ++k) {
+            const int base = bt_rhs(P, (d.t0 + (long)k * gridDim.x - P.tile0) * BT_BLOCK + 32 * w);
+            for (int j = lane; j < nr; j += 32) {
+                df64 s = 0;
+                for (int l = j < base ? j - base + nr : j - base; l < 32; l += nr) s = s + wv[w][k][l];
+                wacc[w][P.slot0 + j] = wacc[w][P.slot0 + j] + s;
+            }
+        }
+    } else {
+        const int G = 32 / nr, g = lane / nr, j = lane - g * nr;
+        df64 acc = lane < nr ? wacc[w][P.slot0 + lane] : df64(0.0f, 0.0f);
+        for (int k0 = 0; k0 < d.n; k0 += G) {
+            const int k = k0 + g;
+            df64 s = 0;
+            if (g < G && k < d.n) {
+                const int base =
+                    bt_rhs(P, (d.t0 + (long)k * gridDim.x - P.tile0) * BT_BLOCK + 32 * w);
+                for (int l = j < base ? j - base + nr : j - base; l < 32; l += nr)
+                    s = s + wv[w][k][l];
+            }
+            const int left = d.n - k0 < G ? d.n - k0 : G;
+            for (int i = 0; i < left; ++i) {
+                const int from = i * nr + (lane < nr ? lane : 0);
+                acc = acc + df64(__shfl_sync(0xffffffffu, s.hi, from),
+                                 __shfl_sync(0xffffffffu, s.lo, from));
+            }
+        }
+        if (lane < nr) wacc[w][P.slot0 + lane] = acc;
+    }
+    __syncwarp();
+    d.n = 0;
+}
+// keep the warp's values v of tile t of problem prob
+__device__ __forceinline__ void bt_defer(const BtArgs &a, BtDeferred &d, int prob, long t, df64 v,
+                                         df64 (*wv)[BT_DEFER][32], df64 (*wacc)[BT_MAX_SLOTS]) {
+    if (d.n == BT_DEFER || (d.n > 0 && d.prob != prob)) bt_flush(a, d, wv, wacc);
+    if (d.n == 0) {
+        d.t0 = t;
+        d.prob = prob;
+    }
+    wv[threadIdx.x >> 5][d.n][threadIdx.x & 31] = v;
+    ++d.n;
 }
 
 template <int BLOCK = BT_BLOCK>
@@ -360,11 +432,10 @@ __device__ __forceinline__ void bt_warp_sums2(df64 v0, df64 v1, const BtProb &P,
     wv[2 * threadIdx.x + 1] = v1;
     __syncwarp();
     const int nr = P.nrhs;
-    const long iw = item0 + 64 * w;
-    const int base = (int)(iw % nr);
+    const int base = bt_rhs(P, item0 + 64 * w);
     for (int j = lane; j < nr; j += 32) {
         df64 s = 0;
-        for (int l = (j - base + nr) % nr; l < 64; l += nr) s = s + wv[64 * w + l];
+        for (int l = j < base ? j - base + nr : j - base; l < 64; l += nr) s = s + wv[64 * w + l];
         wacc[w][P.slot0 + j] = wacc[w][P.slot0 + j] + s;
     }
     __syncwarp();
