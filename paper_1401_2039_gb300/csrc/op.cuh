@@ -101,3 +101,13 @@ struct wd_op {
     size_t hi_field_bytes() const { return wd::field_bytes(hi_prec, g.stride, 24); }
 };
 
+// The handle's own stream and operator for solvers that keep their fields in
+// the storage layout of the operator (wd_api.cu): op_fork makes op->stream wait
+// for the caller's stream, op_join the reverse; op_hop and op_schur queue
+// out = H in and out = Mhat_p in (dagger: Mhat_p^dag) on op->stream.
+namespace wd {
+int op_fork(wd_op *op);
+int op_join(wd_op *op);
+int op_hop(wd_op *op, int out_parity, int dagger, void *out, const void *in);
+int op_schur(wd_op *op, int parity, int dagger, void *out, const void *in);
+}  // namespace wd

@@ -150,6 +150,20 @@ static int check_op(const wd_op *op) {
     return WD_OK;
 }
 
+namespace wd {
+int op_fork(wd_op *op) {
+    WD_TRY(check_op(op));
+    return fork(op);
+}
+int op_join(wd_op *op) { return join(op); }
+int op_hop(wd_op *op, int out_parity, int dagger, void *out, const void *in) {
+    return dslash(op, false, out_parity, dagger, out, in, nullptr, 1.0, nullptr);
+}
+int op_schur(wd_op *op, int parity, int dagger, void *out, const void *in) {
+    return schur(op, false, parity, dagger, out, in, op->ftmp, nullptr);
+}
+}  // namespace wd
+
 // Autotuner: time every launch configuration of one hopping-term variant on
 // this operator's lattice (two warm-up and five timed launches each, CUDA
 // events on the work stream) and keep the fastest.  Variant 0: the plain

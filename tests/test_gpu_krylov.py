@@ -157,3 +157,19 @@ def test_initial_guess_limits_and_bad_operator():
     lo.close()
     kr.close()
     op.close()
+
+
+@pytest.mark.parametrize("method", METHODS)
+@pytest.mark.parametrize("dims,parity", [((12, 12, 12, 8), 1), ((14, 10, 6, 18), 0)])
+def test_lattices_beyond_one_sweep_of_the_grid(method, dims, parity):
+    """More sites than the vector kernels' grid covers at once, against CGNR of
+    the operator: residuals of at most 1e-10 and a spectrum within 1 +- 8 kappa
+    leave the solutions within 2e-10 * 1.8 / 0.2 = 1.8e-9."""
+    U = syn.su3_links(dims, eps=0.3, seed=33)
+    b = cuda(syn.gaussian_spinor(syn.volume(dims), 34))
+    op, kr = make(dims, 0.1, U, method)
+    want = op.solve(b, tol=1e-10).x
+    for _ in range(2):   # the second on the state that the first leaves
+        res = kr.solve(b, tol=1e-10, parity=parity)
+        assert res.status == 0 and res.info["true_rel_resid"] <= 1e-10
+        assert float((res.x - want).norm() / want.norm()) < 1.8e-9
