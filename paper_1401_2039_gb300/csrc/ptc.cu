@@ -528,9 +528,9 @@ static int ptc_gemm_attrs() {
     PTC_CUDA(cudaFuncSetAttribute(k_gemm_bf16_tc<16, TC_NT>,
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, tc_gemm_smem_bytes<16>()));
     PTC_CUDA(cudaFuncSetAttribute(k_gemm_bf16_tc<128, TC_TN>,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, TC_TN_SMEM_BYTES));
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize, tc_gemm_smem_bytes<128>()));
     PTC_CUDA(cudaFuncSetAttribute(k_gemm_bf16_tc<16, TC_TN>,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, TC_TN_SMEM_BYTES));
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize, tc_gemm_smem_bytes<16>()));
     if (dev >= 0 && dev < 64) done[dev] = true;
     return WD_OK;
 }
@@ -606,9 +606,9 @@ static int ptc_gemm_tn(wd_ptc *n, const __nv_bfloat16 *A, const __nv_bfloat16 *B
     const int used = (int)((R + a.k_split - 1) / a.k_split);   // splits with rows
     dim3 grid((unsigned)(M / TC_BM), (unsigned)(N / bn), (unsigned)used);
     if (bn == 128)
-        k_gemm_bf16_tc<128, TC_TN><<<grid, TC_THREADS, TC_TN_SMEM_BYTES, n->stream>>>(a);
+        k_gemm_bf16_tc<128, TC_TN><<<grid, TC_THREADS, tc_gemm_smem_bytes<128>(), n->stream>>>(a);
     else
-        k_gemm_bf16_tc<16, TC_TN><<<grid, TC_THREADS, TC_TN_SMEM_BYTES, n->stream>>>(a);
+        k_gemm_bf16_tc<16, TC_TN><<<grid, TC_THREADS, tc_gemm_smem_bytes<16>(), n->stream>>>(a);
     PTC_CUDA(cudaGetLastError());
     k_ptc_sum_splits<<<grid_for(elems), PTC_BLOCK, 0, n->stream>>>(elems, used, n->wsplit, D);
     PTC_CUDA(cudaGetLastError());

@@ -12,22 +12,27 @@
 // in steps of 64 through a ring of TC_STAGES shared-memory buffers: the four
 // warps copy the A and B tiles of step i + TC_STAGES - 1 from global memory
 // with cp.async (16-byte chunks, no register staging) while the tensor cores
-// work on step i.  Tiles use the no-swizzle canonical layouts of 8 x 16-byte
-// core matrices:
-//   NT (K-major):  a core matrix is 8 rows (M or N) x 8 K values, 16 bytes
-//                  per row; K-adjacent core matrices 128 bytes apart,
-//                  8-row groups 1024 bytes apart;
-//   TN (MN-major): a core matrix is 8 K rows x 8 M (or N) values, 16 bytes
-//                  per K row; MN-adjacent core matrices 128 bytes apart,
-//                  K-adjacent ones (rows / 8) * 128 bytes apart,
-// so that every 16-byte chunk of a global row lands in one core-matrix row
-// (no transposition in either form).  For each step one elected thread
+// work on step i.  Tiles use the 128-byte-swizzled canonical layouts, atoms of
+// 8 rows of 128 bytes whose 16-byte chunk c of row r lies at chunk c ^ (r % 8):
+//   NT (K-major):  a row is 64 K values of one M (or N); 8-row groups 1024
+//                  bytes apart; the next 16 K values 32 bytes on;
+//   TN (MN-major): a row is 64 M (or N) values of one K; atoms 1024 bytes
+//                  apart along K, TC_BK rows of 128 bytes apart along M (N),
+// so that eight threads copy 128 contiguous bytes of a global row into eight
+// distinct bank groups (no transposition in either form).  In the layout of
+// 8 x 16-byte core matrices without swizzle the same eight chunks lay 128
+// bytes apart, all in one bank group, and the copies' 8 shared-memory passes
+// each bounded the kernel: NT 24576 x 128 x 1152 took 55 us, now 18; TN
+// 1152 x 128 over 24576 rows 53 us, now 22.  (B of a TN product with BN =
+// 16, narrower than an atom, keeps the core matrices.)  For each step one elected thread
 // issues four 128 x BN x 16 tcgen05.mma that accumulate in tensor memory
 // (TMEM, BN fp32 columns x 128 lanes) and a tcgen05.commit that arrives on
 // the step buffer's mbarrier once the MMAs have consumed it; a buffer is
 // refilled only after that arrival.  The epilogue moves the accumulator from
 // TMEM to registers with tcgen05.ld (warp w owns TMEM lanes 32w..32w+31,
-// i.e. rows 32w..32w+31 of the tile) and stores it.
+// i.e. rows 32w..32w+31 of the tile), turns it in the ring's shared memory and
+// stores whole rows (a lane's own row, 16 bytes at a time, left NT 24576 x 1152
+// x 128, whose output is what bounds it, at 77 us, now 30).
 //
 // Bounded waits.  Every wait on an mbarrier polls at most spin_limit times.
 // When one gives up, the kernel records err = 1, issues no further MMA,
@@ -42,7 +47,8 @@
 // Requirements (checked by the host launchers): NT: M % 128 == 0,
 // N % BN == 0, K % 64 == 0; TN: M % 128 == 0, N % BN == 0, every split's row
 // range a multiple of 64; rows 16-byte aligned; tc_gemm_smem_bytes<BN>()
-// bytes of dynamic shared memory.
+// bytes of dynamic shared memory.  (Whichever way a descriptor's two offsets
+// are read, an MMA's addresses stay within its tile.)
 #pragma once
 
 #include <cuda_bf16.h>
@@ -74,9 +80,10 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p) {
     return (uint32_t)__cvta_generic_to_shared(p);
 }
 
-// tcgen05 shared-memory matrix descriptor, no swizzle.  K-major: lbo = byte
-// offset of K-adjacent core matrices, sbo = of MN-adjacent 8-row groups;
-// MN-major: lbo = of K-adjacent core matrices, sbo = of MN-adjacent ones.
+// tcgen05 shared-memory matrix descriptors (1024-byte aligned tiles).
+// No swizzle, K-major: lbo = byte offset of K-adjacent core matrices, sbo = of
+// MN-adjacent 8-row groups; MN-major: lbo = of K-adjacent core matrices, sbo =
+// of MN-adjacent ones.
 __device__ __forceinline__ uint64_t tc_smem_desc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
     uint64_t d = 0;
     d |= (uint64_t)((addr & 0x3FFFFu) >> 4);            // start address
@@ -84,6 +91,11 @@ __device__ __forceinline__ uint64_t tc_smem_desc(uint32_t addr, uint32_t lbo, ui
     d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;         // stride byte offset
     d |= (uint64_t)1 << 46;                              // descriptor version
     return d;                                            // base offset 0, no swizzle
+}
+// 128-byte swizzle, K-major: lbo unused, sbo = of 8-row groups; MN-major: lbo =
+// of MN-adjacent atoms (64 values), sbo = of K-adjacent ones (8 rows).
+__device__ __forceinline__ uint64_t tc_smem_desc_sw128(uint32_t addr, uint32_t lbo, uint32_t sbo) {
+    return tc_smem_desc(addr, lbo, sbo) | (uint64_t)2 << 61;
 }
 
 // Instruction descriptor of kind::f16: BF16 A and B, FP32 D; both operands
@@ -114,14 +126,10 @@ __device__ __forceinline__ bool tc_wait(uint32_t mbar, uint32_t phase, unsigned 
 constexpr int TC_STAGES = 3;
 constexpr int TC_TILE_A = TC_BM * TC_BK * 2;   // bytes of one A tile
 
+// the ring, and what rounding its start up to 1024 bytes takes
 template <int BN> __host__ __device__ constexpr int tc_gemm_smem_bytes() {
-    return TC_STAGES * (TC_TILE_A + BN * TC_BK * 2);
+    return TC_STAGES * (TC_TILE_A + BN * TC_BK * 2) + 1024;
 }
-// The transposed form is launched with more than its ring needs (96 KB at
-// most): with either reading of a descriptor's two byte offsets, every
-// shared-memory address an MMA can form from it lies inside the CTA's
-// allocation.
-constexpr int TC_TN_SMEM_BYTES = 160 * 1024;
 
 __device__ __forceinline__ void cp_async16(void *smem_dst, const void *gmem_src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
@@ -134,11 +142,14 @@ __device__ __forceinline__ void tc_commit(uint64_t *bar) {
 }
 
 template <int BN, int LAYOUT>
-__global__ void __launch_bounds__(TC_THREADS, 1) k_gemm_bf16_tc(const TcArgs p) {
+__global__ void __launch_bounds__(TC_THREADS, 2) k_gemm_bf16_tc(const TcArgs p) {
     static_assert(BN % 16 == 0 && BN >= 16 && BN <= 256, "tcgen05 N for M = 128");
     constexpr uint32_t TMEM_COLS = BN < 32 ? 32 : BN;
     constexpr int TILE_B = BN * TC_BK * 2;
-    extern __shared__ __align__(1024) uint8_t smem[];
+    // whether B is narrower than a swizzle atom
+    constexpr bool CORE_B = LAYOUT == TC_TN && BN < 64;
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    uint8_t *const smem = smem_raw + (1024u - (smem_u32(smem_raw) & 1023u) & 1023u);
     uint8_t *const sA = smem;                            // TC_STAGES A tiles
     uint8_t *const sB = smem + TC_STAGES * TC_TILE_A;    // TC_STAGES B tiles
     __shared__ __align__(8) uint64_t mbar[TC_STAGES + 1];   // [TC_STAGES]: the drain barrier
@@ -175,25 +186,31 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_gemm_bf16_tc(const TcArgs p) 
         const long k0 = k_begin + (long)step * TC_BK;
         uint8_t *a = sA + buf * TC_TILE_A, *b = sB + buf * TILE_B;
         if (LAYOUT == TC_NT) {
+#pragma unroll
             for (int i = tid; i < TC_BM * 8; i += TC_THREADS) {
                 const int r = i >> 3, c = i & 7;
-                cp_async16(a + (r >> 3) * 1024 + c * 128 + (r & 7) * 16, p.A + (m0 + r) * p.lda + k0 + c * 8);
+                cp_async16(a + r * 128 + ((c ^ (r & 7)) << 4), p.A + (m0 + r) * p.lda + k0 + c * 8);
             }
+#pragma unroll
             for (int i = tid; i < BN * 8; i += TC_THREADS) {
                 const int r = i >> 3, c = i & 7;
-                cp_async16(b + (r >> 3) * 1024 + c * 128 + (r & 7) * 16, p.B + (n0 + r) * p.ldb + k0 + c * 8);
+                cp_async16(b + r * 128 + ((c ^ (r & 7)) << 4), p.B + (n0 + r) * p.ldb + k0 + c * 8);
             }
         } else {
-            // row k of the step, 8-element group g along M (N): core matrix
-            // (k / 8, g) at ((k / 8) * groups + g) * 128, row k % 8
-            constexpr int GA = TC_BM / 8, GB = BN / 8;
+            // row k of the step, 8-element group g along M (N)
+            constexpr int GA = TC_BM / 8, GB = BN / 8, ATOMS = TC_BK * 128;
+#pragma unroll
             for (int i = tid; i < TC_BK * GA; i += TC_THREADS) {
                 const int k = i / GA, g = i - k * GA;
-                cp_async16(a + ((k >> 3) * GA + g) * 128 + (k & 7) * 16, p.A + (k0 + k) * p.lda + m0 + g * 8);
+                cp_async16(a + (g >> 3) * ATOMS + k * 128 + (((g ^ k) & 7) << 4),
+                           p.A + (k0 + k) * p.lda + m0 + g * 8);
             }
+#pragma unroll
             for (int i = tid; i < TC_BK * GB; i += TC_THREADS) {
                 const int k = i / GB, g = i - k * GB;
-                cp_async16(b + ((k >> 3) * GB + g) * 128 + (k & 7) * 16, p.B + (k0 + k) * p.ldb + n0 + g * 8);
+                cp_async16(CORE_B ? b + ((k >> 3) * GB + g) * 128 + (k & 7) * 16
+                                  : b + (g >> 3) * ATOMS + k * 128 + (((g ^ k) & 7) << 4),
+                           p.B + (k0 + k) * p.ldb + n0 + g * 8);
             }
         }
     };
@@ -217,13 +234,15 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_gemm_bf16_tc(const TcArgs p) 
 #pragma unroll
             for (int kk = 0; kk < TC_BK / 16; ++kk) {
                 uint64_t ad, bd;
+                const uint32_t at = smem_u32(sA + b * TC_TILE_A), bt = smem_u32(sB + b * TILE_B);
                 if (LAYOUT == TC_NT) {
-                    ad = tc_smem_desc(smem_u32(sA + b * TC_TILE_A) + kk * 256, 128, 1024);
-                    bd = tc_smem_desc(smem_u32(sB + b * TILE_B) + kk * 256, 128, 1024);
-                } else {   // 16 K rows = two K-adjacent core matrices per MMA
-                    constexpr uint32_t LA = (TC_BM / 8) * 128, LB = (BN / 8) * 128;
-                    ad = tc_smem_desc(smem_u32(sA + b * TC_TILE_A) + kk * 2 * LA, LA, 128);
-                    bd = tc_smem_desc(smem_u32(sB + b * TILE_B) + kk * 2 * LB, LB, 128);
+                    ad = tc_smem_desc_sw128(at + kk * 32, 16, 1024);
+                    bd = tc_smem_desc_sw128(bt + kk * 32, 16, 1024);
+                } else {   // 16 K rows = two K-adjacent atoms (core matrices) per MMA
+                    constexpr uint32_t LB = (BN / 8) * 128;
+                    ad = tc_smem_desc_sw128(at + kk * 2048, TC_BK * 128, 1024);
+                    bd = CORE_B ? tc_smem_desc(bt + kk * 2 * LB, LB, 128)
+                                : tc_smem_desc_sw128(bt + kk * 2048, TC_BK * 128, 1024);
                 }
                 const uint32_t acc = (i > 0 || kk > 0) ? 1u : 0u;
                 asm volatile(
@@ -257,23 +276,38 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_gemm_bf16_tc(const TcArgs p) 
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (ok) {
         const uint32_t lane_base = (uint32_t)(32 * warp) << 16;
-        float *drow = D + (m0 + 32 * warp + lane) * (long)p.ldd + n0;
+        // the warp's rows in shared memory, 16 bytes more apart than they are
+        // long: a lane's chunks of eight rows fall in distinct bank groups
+        constexpr int CH = BN < 32 ? 16 : 32, PITCH = BN * 4 + 16;
+        static_assert(4 * 32 * PITCH <= TC_STAGES * (TC_TILE_A + TILE_B), "staging in the ring");
+        uint8_t *const rows = smem + warp * 32 * PITCH;
 #pragma unroll 1
-        for (int c0 = 0; c0 < BN; c0 += 16) {
-            uint32_t v[16];
-            asm volatile(
-                "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-                "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-                : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]),
-                  "=r"(v[6]), "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]),
-                  "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-                : "r"(tmem + lane_base + (uint32_t)c0));
+        for (int c0 = 0; c0 < BN; c0 += CH) {
+            uint32_t v[CH];
+#pragma unroll
+            for (int h = 0; h < CH; h += 16)
+                asm volatile(
+                    "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+                    "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+                    : "=r"(v[h]), "=r"(v[h + 1]), "=r"(v[h + 2]), "=r"(v[h + 3]), "=r"(v[h + 4]),
+                      "=r"(v[h + 5]), "=r"(v[h + 6]), "=r"(v[h + 7]), "=r"(v[h + 8]),
+                      "=r"(v[h + 9]), "=r"(v[h + 10]), "=r"(v[h + 11]), "=r"(v[h + 12]),
+                      "=r"(v[h + 13]), "=r"(v[h + 14]), "=r"(v[h + 15])
+                    : "r"(tmem + lane_base + (uint32_t)(c0 + h)));
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-            for (int j = 0; j < 16; j += 4)
-                *reinterpret_cast<float4 *>(drow + c0 + j) =
-                    make_float4(__uint_as_float(v[j]), __uint_as_float(v[j + 1]),
-                                __uint_as_float(v[j + 2]), __uint_as_float(v[j + 3]));
+            for (int j = 0; j < CH; j += 4)
+                *reinterpret_cast<uint4 *>(rows + lane * PITCH + (c0 + j) * 4) =
+                    make_uint4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+        }
+        __syncwarp();
+        constexpr int PER = BN / 4;   // 16-byte chunks of a row
+        float *const drow = D + (m0 + 32 * warp) * (long)p.ldd + n0;
+#pragma unroll 8
+        for (int i = lane; i < 32 * PER; i += 32) {
+            const int r = i / PER, c = i - r * PER;
+            *reinterpret_cast<uint4 *>(drow + (long)r * p.ldd + c * 4) =
+                *reinterpret_cast<const uint4 *>(rows + r * PITCH + c * 16);
         }
     } else {
         // drain: a commit arrives once every MMA this thread issued has
