@@ -173,6 +173,66 @@ k_ptc_gather(PtcGeom g, int cin, const float *__restrict__ F, int ldf,
     }
 }
 
+// The same for one input channel (every network's first layer): one thread per
+// (site x, transport k), and a block turns the rows of A of its 16 sites in
+// shared memory, so that they go out whole.  The kernel above has no channels
+// to spread over a warp there and stores 8 bytes at a time, 768 apart: 16^3 x 32
+// took 104 us, now 60, bound by the scattered reads of links and spinors.  With
+// 16 channels this form takes longer (36 us against 20 on 8^3 x 16: nine times
+// the site arithmetic).
+constexpr int PTC_GATHER1_SITES = 16;
+__global__ void __launch_bounds__(PTC_NK * PTC_GATHER1_SITES)
+k_ptc_gather1(PtcGeom g, const float *__restrict__ F, int ldf, const float2 *__restrict__ U,
+              __nv_bfloat16 *__restrict__ A, int lda) {
+    constexpr int K = 36;
+    __shared__ __align__(16) __nv_bfloat16 rows[PTC_GATHER1_SITES * 3 * 2 * K];   // [site][a][2 K]
+    const long x0 = (long)blockIdx.x * PTC_GATHER1_SITES;
+    const int n = (int)(g.V - x0 < PTC_GATHER1_SITES ? g.V - x0 : PTC_GATHER1_SITES);
+    const int xs = threadIdx.x / PTC_NK, k = threadIdx.x - xs * PTC_NK;
+    if (xs < n) {
+        const long x = x0 + xs;
+        float2 v[3][4];
+        if (k == 0) {
+            for (int a = 0; a < 3; ++a) load_spins(F + (x * 3 + a) * (long)ldf, 1, 0, v[a]);
+        } else {
+            int co[4];
+            lex_coords(g, x, co);
+            const int mu = (k - 1) & 3;
+            const bool fwd = k <= 4;
+            bool wrap;
+            const long xn = ptc_neighbour(g, co, mu, fwd ? 1 : -1, wrap);
+            float2 p[3][4];
+            for (int b = 0; b < 3; ++b) load_spins(F + (xn * 3 + b) * (long)ldf, 1, 0, p[b]);
+            const float2 *Ul = U + ((fwd ? x : xn) * 4 + mu) * 9;
+            float pr = 1.f, pi = 0.f;
+            if (wrap) { pr = g.ph[2 * mu]; pi = fwd ? g.ph[2 * mu + 1] : -g.ph[2 * mu + 1]; }
+            for (int a = 0; a < 3; ++a)
+                for (int s = 0; s < 4; ++s) {
+                    float re = 0.f, im = 0.f;
+                    for (int b = 0; b < 3; ++b) {
+                        // forward: U[a][b]; backward: conj(U[b][a])
+                        const float2 u = fwd ? Ul[3 * a + b] : Ul[3 * b + a];
+                        const float ui = fwd ? u.y : -u.y;
+                        re += u.x * p[b][s].x - ui * p[b][s].y;
+                        im += u.x * p[b][s].y + ui * p[b][s].x;
+                    }
+                    v[a][s] = make_float2(re * pr - im * pi, re * pi + im * pr);
+                }
+        }
+        for (int a = 0; a < 3; ++a) {
+            __nv_bfloat16 *row = rows + (xs * 3 + a) * 2 * K + k * 4;
+            store_bf16x4(row, v[a][0].x, v[a][1].x, v[a][2].x, v[a][3].x);
+            store_bf16x4(row + K, v[a][0].y, v[a][1].y, v[a][2].y, v[a][3].y);
+        }
+    }
+    __syncthreads();
+    constexpr int per = K / 4;   // 16-byte chunks of a row
+    for (int i = threadIdx.x; i < n * 3 * per; i += PTC_NK * PTC_GATHER1_SITES) {
+        const int r = i / per, q = i - r * per;
+        reinterpret_cast<uint4 *>(A + (x0 * 3 + r) * lda)[q] = reinterpret_cast<const uint4 *>(rows)[i];
+    }
+}
+
 // Real block form of the complex weights: B[(p', c', s')][(p, k, c, s)], row
 // stride ldb, from W (complex64 as float2) [cout][cin][9][4][4].
 __global__ void k_ptc_weights(int cout, int cin, const float2 *__restrict__ W,
@@ -272,24 +332,31 @@ __global__ void k_ptc_loss_grad(long V, const float *__restrict__ F, int ld,
 
 // Adjoint of the gather: dF_c(x) = sum_k (T_k^dag dA_{c,k})(x) with
 // T_{1+mu}^dag = T_{5+mu} and T_{5+mu}^dag = T_{1+mu}; dA rows (y, a) hold
-// [Re (k, c, s)][Im (k, c, s)].  One thread per (site x, channel c).
+// [Re (k, c, s)][Im (k, c, s)].  One thread per (site x, channel c, pair of
+// spins): a warp's loads are contiguous, and 16 channels on 8^3 x 16 make 84 %
+// of the threads that the chip holds.  Bound by dA (113 MB there); one thread
+// per (x, c), a number at a time, took 40 us, now 31.
 __global__ void __launch_bounds__(PTC_BLOCK)
 k_ptc_scatter(PtcGeom g, int cin, const float *__restrict__ dA, int lda,
               const float2 *__restrict__ U, float *__restrict__ dF, int ldf,
               __nv_bfloat16 *__restrict__ dFb, int ldfb) {
     const long t = (long)blockIdx.x * PTC_BLOCK + threadIdx.x;
-    if (t >= g.V * cin) return;
-    const long x = t / cin;
-    const int c = (int)(t - x * cin);
+    if (t >= g.V * cin * 2) return;
+    const long x = t / (2 * cin);
+    const int c2 = (int)(t - x * 2 * cin) * 2;   // 4 c + first spin
     int co[4];
     lex_coords(g, x, co);
     const int K = cin * 36;
-    float2 acc[3][4];
-    for (int a = 0; a < 3; ++a)
-        for (int s = 0; s < 4; ++s) {
-            const float *row = dA + (x * 3 + a) * (long)lda + c * 4;
-            acc[a][s] = make_float2(row[s], row[K + s]);
-        }
+    float2 acc[3][2];
+    auto load = [&](const float *row, float2 v[2]) {   // two spins of a channel
+        const float2 re = *reinterpret_cast<const float2 *>(row);
+        const float2 im = *reinterpret_cast<const float2 *>(row + K);
+        v[0] = make_float2(re.x, im.x);
+        v[1] = make_float2(re.y, im.y);
+    };
+#pragma unroll
+    for (int a = 0; a < 3; ++a) load(dA + (x * 3 + a) * (long)lda + c2, acc[a]);
+#pragma unroll 2
     for (int k = 1; k < PTC_NK; ++k) {
         const int mu = (k - 1) & 3;
         // dA_{c,k} is transported by T_k^dag: backward hop for k <= 4, forward otherwise
@@ -299,15 +366,15 @@ k_ptc_scatter(PtcGeom g, int cin, const float *__restrict__ dA, int lda,
         const float2 *Ul = U + ((fwd ? x : xn) * 4 + mu) * 9;
         float pr = 1.f, pi = 0.f;
         if (wrap) { pr = g.ph[2 * mu]; pi = fwd ? g.ph[2 * mu + 1] : -g.ph[2 * mu + 1]; }
-        float2 p[3][4];
-        for (int b = 0; b < 3; ++b)
-            for (int s = 0; s < 4; ++s) {
-                const float *row = dA + (xn * 3 + b) * (long)lda + (k * cin + c) * 4;
-                p[b][s] = make_float2(row[s], row[K + s]);
-            }
+        float2 p[3][2];
+#pragma unroll
+        for (int b = 0; b < 3; ++b) load(dA + (xn * 3 + b) * (long)lda + k * cin * 4 + c2, p[b]);
+#pragma unroll
         for (int a = 0; a < 3; ++a)
-            for (int s = 0; s < 4; ++s) {
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
                 float re = 0.f, im = 0.f;
+#pragma unroll
                 for (int b = 0; b < 3; ++b) {
                     const float2 u = fwd ? Ul[3 * a + b] : Ul[3 * b + a];
                     const float ui = fwd ? u.y : -u.y;
@@ -318,15 +385,15 @@ k_ptc_scatter(PtcGeom g, int cin, const float *__restrict__ dA, int lda,
                 acc[a][s].y += re * pi + im * pr;
             }
     }
+#pragma unroll
     for (int a = 0; a < 3; ++a) {
-        float *row = dF + (x * 3 + a) * (long)ldf;
-        __nv_bfloat16 *rb = dFb + (x * 3 + a) * (long)ldfb;
-        for (int s = 0; s < 4; ++s) {
-            row[c * 4 + s] = acc[a][s].x;
-            row[4 * cin + c * 4 + s] = acc[a][s].y;
-            rb[c * 4 + s] = __float2bfloat16_rn(acc[a][s].x);
-            rb[4 * cin + c * 4 + s] = __float2bfloat16_rn(acc[a][s].y);
-        }
+        float *row = dF + (x * 3 + a) * (long)ldf + c2;
+        __nv_bfloat16 *rb = dFb + (x * 3 + a) * (long)ldfb + c2;
+        *reinterpret_cast<float2 *>(row) = make_float2(acc[a][0].x, acc[a][1].x);
+        *reinterpret_cast<float2 *>(row + 4 * cin) = make_float2(acc[a][0].y, acc[a][1].y);
+        *reinterpret_cast<__nv_bfloat162 *>(rb) = __floats2bfloat162_rn(acc[a][0].x, acc[a][1].x);
+        *reinterpret_cast<__nv_bfloat162 *>(rb + 4 * cin) =
+            __floats2bfloat162_rn(acc[a][0].y, acc[a][1].y);
     }
 }
 
@@ -696,8 +763,13 @@ static int ptc_forward(wd_ptc *n, const double *r, double in_scale, bool keep_op
             PTC_TRY(ptc_layer_fused(n, l));
             continue;
         }
-        k_ptc_gather<<<grid_for(V * cin), PTC_BLOCK, 0, n->stream>>>(n->g, cin, n->F[l], n->ldF[l],
-                                                                      n->U, n->A[l], n->Kp[l]);
+        if (cin == 1)
+            k_ptc_gather1<<<(unsigned)((V + PTC_GATHER1_SITES - 1) / PTC_GATHER1_SITES),
+                            PTC_NK * PTC_GATHER1_SITES, 0, n->stream>>>(n->g, n->F[l], n->ldF[l],
+                                                                        n->U, n->A[l], n->Kp[l]);
+        else
+            k_ptc_gather<<<grid_for(V * cin), PTC_BLOCK, 0, n->stream>>>(
+                n->g, cin, n->F[l], n->ldF[l], n->U, n->A[l], n->Kp[l]);
         PTC_CUDA(cudaGetLastError());
         PTC_TRY(ptc_gemm(n, n->A[l], n->B[l], n->F[l + 1], n->Mp, n->Np[l], n->Kp[l], n->Kp[l],
                          n->Kp[l], n->ldF[l + 1]));
@@ -882,7 +954,7 @@ static int ptc_accumulate(wd_ptc *n, const double *r, const double *e, int ns, d
             // dA = dF[l+1] B[l] on the tensor cores, then the adjoint transports
             PTC_TRY(ptc_gemm(n, n->dFb[l + 1], n->Bt[l], n->dA, n->Mp, n->Kp[l], n->Rp[l + 1],
                              n->Rp[l + 1], n->Rp[l + 1], n->Kp[l]));
-            k_ptc_scatter<<<grid_for(V * n->ch[l]), PTC_BLOCK, 0, n->stream>>>(
+            k_ptc_scatter<<<grid_for(V * n->ch[l] * 2), PTC_BLOCK, 0, n->stream>>>(
                 n->g, n->ch[l], n->dA, n->Kp[l], n->U, n->dF[l], n->ldF[l], n->dFb[l], n->Rp[l]);
             PTC_CUDA(cudaGetLastError());
         }
