@@ -59,8 +59,42 @@ __global__ void __launch_bounds__(FX_BLOCK, 5) k_dslash_fx(const __grid_constant
 }
 
 template <int EPI, int NORM>
+__global__ void __launch_bounds__(FXW_BLOCK, 1) k_dslash_fx_wide(const __grid_constant__ FxArgs A) {
+    __shared__ FxWideShared sh;
+    const DslashArgs<double> &a = A.d;
+    const int lane = threadIdx.x & 31, w = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);
+    const long hs = a.h0 + (long)blockIdx.x * FX_SITES + lane;
+    const long h = hs < a.h1 ? hs : a.h1 - 1;
+    double v[2];
+    fx_site_wide(A, (unsigned)h, w, sh, v);
+    double sq = 0;
+    if (w < 12 && hs < a.h1) {
+        const double2 o = fx_store<EPI>(a, h, w >> 2, w & 3, v[0], v[1]);
+        if (NORM) sq = o.x * o.x + o.y * o.y;
+    }
+    if (NORM) {
+        __shared__ df64 ws[12][32];
+        if (w < 12) ws[w][lane] = to_df(sq);
+        __syncthreads();
+        if (w == 0) {
+            df64 t = ws[0][lane];
+#pragma unroll
+            for (int j = 1; j < 12; ++j) t = t + ws[j][lane];
+            t = warp_sum(t);
+            if (lane == 0) a.red.partials[blockIdx.x] = t;
+        }
+    }
+}
+
+template <int EPI, int NORM>
 void launch_fx(const FxArgs &A, cudaStream_t s) {
     const long n = A.d.h1 - A.d.h0;
+    // By the lattice, not by the launch's range of sites, so that a hop in parts
+    // rounds as a whole one.
+    if ((A.d.g.vh + FX_SITES - 1) / FX_SITES <= FXW_MAX_BLOCKS) {
+        k_dslash_fx_wide<EPI, NORM><<<(unsigned)((n + FX_SITES - 1) / FX_SITES), FXW_BLOCK, 0, s>>>(A);
+        return;
+    }
     k_dslash_fx<EPI, NORM><<<(unsigned)((n + FX_SITES - 1) / FX_SITES), FX_BLOCK, 0, s>>>(A);
 }
 

@@ -440,4 +440,98 @@ __device__ __forceinline__ void fx_site(const FxArgs &A, unsigned h, int w, FxSh
     }
 }
 
+// The same with one hop per warp, for lattices whose blocks leave the chip nearly
+// empty: there a launch is a warp's chain of four hops, on four warps per SM.
+// Sixteen warps take 32 sites, warp w = 4 mu + 2 backward + k row k of one hop,
+// and leave the product and its exponent in shared memory; then twelve warps
+// each add the eight terms of one complex number j = 4 colour + spin, in units
+// of the largest exponent.
+//
+// A hop, with the host's share, one warp per row and sense / one per hop:
+//   blocks    4 (4^4)   64 (8^4)   128 (8^3 x 16)   192   324 (12^4)   2048
+//   us     10.9 / 8.0  11.0 / 8.7    11.3 / 8.7   13.2 / 13.0  14.8 / 17.7  42 / 67
+// so the line lies where one block per SM ends; a block of 16 warps with 128
+// registers leaves no room for a second.
+constexpr int FXW_BLOCK = 512;
+constexpr long FXW_MAX_BLOCKS = 152;
+
+struct FxWideShared {
+    long long u[16][6][32];
+    int xa[16][32];      // exponent, negative: no term, 1 << 24: a bad site
+};
+
+// v = complex number w (w < 12) of H in at site h, [re, im]
+__device__ __forceinline__ void fx_site_wide(const FxArgs &A, unsigned h, int w, FxWideShared &sh,
+                                             double v[2]) {
+    const int lane = threadIdx.x & 31;
+    {
+        const int mu = w >> 2, k = w & 1;
+        const bool fwd = (w & 2) == 0;
+        int c[4];
+        site_coords(A.d.g, h, A.d.parity, c);
+        bool wrap;
+        const unsigned hn = fx_neighbour(A.d.g, h, c, mu, fwd, wrap), site = fwd ? h : hn;
+        uint4 U[3][3];
+        fx_links(A, site, mu, fwd, U);
+        const int eu = fx_link_exp(A, __ldg(A.any_exp) != 0, site, mu, fwd);
+        double r[6];
+        fx_half_row(A, hn, mu, k, fwd, r);
+        if (fx_wraps(A, mu, wrap)) fx_phase(A, mu, fwd, r);
+        const int eb = (int)(fx_max(r) >> 20);
+        int xa = eb + eu;
+        if (fx_out_of_range(eb, eu)) {
+            xa = fx_bits(r) != 0 || eu == FX_BAD_EXP ? 1 << 24 : -1;
+        } else {
+            long long u[6];
+            fx_product(U, r, ((unsigned)eb << 20) | 0xFFFFFu, fwd, u);
+#pragma unroll
+            for (int i = 0; i < 6; ++i) sh.u[w][i][lane] = u[i];
+        }
+        sh.xa[w][lane] = xa;
+    }
+    __syncthreads();
+    if (w >= 12) return;
+    const int s = w & 3, cc = w >> 2;
+    int xm = -1;
+#pragma unroll
+    for (int t = 0; t < 16; ++t) xm = max(xm, sh.xa[t][lane]);
+    if (xm == 1 << 24) {
+        double t[24];
+        fx_fallback(A, h, t);
+#pragma unroll
+        for (int j = 0; j < 12; ++j)
+            if (j == w) { v[0] = t[2 * j]; v[1] = t[2 * j + 1]; }
+        return;
+    }
+    xm = -1;
+    int xt[8];
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {   // t = 2 mu + backward
+        const int k = s < 2 ? s : t < 4 ? 3 - s : s - 2;
+        xt[t] = sh.xa[2 * t + k][lane];
+        xm = max(xm, xt[t]);
+    }
+    long long re = 0, im = 0;
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+        if (xt[t] < 0) continue;
+        const int mu = t >> 1, k = s < 2 ? s : t < 4 ? 3 - s : s - 2;
+        const long long ur = sar64(sh.u[2 * t + k][2 * cc][lane], xm - xt[t]);
+        const long long ui = sar64(sh.u[2 * t + k][2 * cc + 1][lane], xm - xt[t]);
+        if (s < 2) {
+            re += ur;
+            im += ui;
+        } else {
+            // -i u (x, z) or u (y, t), with the row's sign; H: backward minus
+            // forward, H^dag the reverse
+            const bool minus = fx_row_neg(mu, k) != ((t & 1) == (A.dagger != 0 ? 1 : 0));
+            const long long br = (mu & 1) ? ur : ui, bi = (mu & 1) ? ui : -ur;
+            re += minus ? -br : br;
+            im += minus ? -bi : bi;
+        }
+    }
+    v[0] = fx_to_double(re, xm);
+    v[1] = fx_to_double(im, xm);
+}
+
 }  // namespace wd
