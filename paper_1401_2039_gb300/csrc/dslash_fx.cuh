@@ -6,7 +6,7 @@
 // bound by that pipe: 1673 us at 32^3 x 64, 558 us at 24^3 x 48, 131 us at
 // 16^3 x 32, 55 us at 4^4.  Here the SU(3) products and the sum over the eight
 // hops run on the integer pipes; FP64 keeps the spin projection (12 additions
-// per hop) and the epilogue: 516, 172, 41 and 11 us.  What bounds it now: issue
+// per hop) and the epilogue: 516, 172, 41 and 8 us.  What bounds it now: issue
 // (46 % active at the 20 warps per SM that 96 registers allow), with the FP64
 // pipe 53 % busy and DRAM at 40 %.
 //
