@@ -99,9 +99,9 @@ void launch_fx(const FxArgs &A, cudaStream_t s) {
 }
 
 // Fixed-point links of one parity from its FP64 records: one thread per (site,
-// direction).  With m = max(max |u|, 0.4 times the largest sum of absolute
-// values of a row's or a column's six reals): eu = 0 for 1/8 < m <= 1 (SU(3):
-// at most 0.98), else the exponent with m in (2^(eu - 1), 2^eu].
+// direction).  With m = max(max |u|, the largest sum of absolute values of a
+// row's or a column's six reals over 2.46): eu = 0 for 1/8 < m <= 1 (SU(3): at
+// most sqrt(6) / 2.46 = 0.9957), else the exponent with m in (2^(eu - 1), 2^eu].
 template <int RECON>
 __global__ void __launch_bounds__(128)
 k_gauge_fx(Geom g, const char *links, size_t dir_bytes, char *fx, size_t fx_dir_bytes,
@@ -119,8 +119,8 @@ k_gauge_fx(Geom g, const char *links, size_t dir_bytes, char *fx, size_t fx_dir_
         const double u = fabs(U[k]);
         finite = finite && isfinite(u);
         mx = fmax(mx, u);
-        row[k / 6] += 0.4 * u;
-        col[(k / 2) % 3] += 0.4 * u;
+        row[k / 6] += u / 2.46;
+        col[(k / 2) % 3] += u / 2.46;
     }
 #pragma unroll
     for (int k = 0; k < 3; ++k) mx = fmax(mx, fmax(row[k], col[k]));
@@ -142,7 +142,7 @@ k_gauge_fx(Geom g, const char *links, size_t dir_bytes, char *fx, size_t fx_dir_
         uint32_t w[4];
 #pragma unroll
         for (int p = 0; p < 2; ++p) {
-            const long long F = eu == FX_BAD_EXP ? 0ll : __double2ll_rn(ldexp(U[2 * e + p], 61 - eu));
+            const long long F = eu == FX_BAD_EXP ? 0ll : __double2ll_rn(ldexp(U[2 * e + p], 62 - eu));
             const int u0 = (int)F;
             w[2 * p] = (uint32_t)u0;
             w[2 * p + 1] = (uint32_t)((F - u0) >> 32);

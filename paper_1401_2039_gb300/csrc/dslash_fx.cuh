@@ -10,21 +10,21 @@
 // (46 % active at the 20 warps per SM that 96 registers allow), with the FP64
 // pipe 53 % busy and DRAM at 40 %.
 //
-// Numbers.  A link element is u = Fu 2^(eu - 61) with a 61-bit integer Fu and
+// Numbers.  A link element is u = Fu 2^(eu - 62) with a 62-bit integer Fu and
 // one exponent eu per link: |u| <= 2^eu, and the absolute values of the six
-// reals of any row or column add to at most 2.5 2^eu (0 for every SU(3) link,
-// whose rows add to at most sqrt(6)).  It is stored as two signed limbs, Fu =
-// u1 2^32 + u0, |u1| <= 2^29, |u0| <= 2^31, converted once when the gauge field
+// reals of any row or column add to at most 2.46 2^eu (eu = 0 for every SU(3)
+// link, whose rows add to at most sqrt(6)).  It is stored as two signed limbs, Fu =
+// u1 2^32 + u0, |u1| <= 2^30, |u0| <= 2^31, converted once when the gauge field
 // is loaded.  The projected half-spinor row of a hop (6 reals, FP64) is
 // converted to 60-bit integers Fh = h1 2^32 + h0, |h1| <= 2^28, with one shared
 // exponent.  Then
 //   sum Fu Fh = 2^64 (sum u1 h1 + 2^-32 sum (u1 h0 + u0 h1)) + ...
 // with two 64-bit accumulators per real sum; the omitted u0 h0 terms are below
-// a quarter of the last place each.  |sum (u1 h0 + u0 h1)| <= 2.5 2^60 + 6 2^59
-// < 2^63, |sum u1 h1| <= 2.5 2^57, and the sum over the eight hops (exponent XA
+// a quarter of the last place each.  |sum (u1 h0 + u0 h1)| <= 2.46 2^61 + 6 2^59
+// < 2^63, |sum u1 h1| <= 2.46 2^58, and the sum over the eight hops (exponent XA
 // of the site's accumulators, raised when a larger hop arrives) stays below
-// 2^62.  The last place of a hop is 2^-57 of twice its largest component: the
-// result is one rounding of a value good to about 2^-56 of the site's scale,
+// 2^63.  The last place of a hop is 2^-58 of twice its largest component: the
+// result is one rounding of a value good to about 2^-57 of the site's scale,
 // where FP64 arithmetic rounds after every operation.  Against 113-bit
 // arithmetic (relative 2-norm, 6 x 10 x 14 x 18): Gaussian fields 7.0e-17 (FP64
 // arithmetic 1.5e-16), fields falling by e^3 per time slice 7.0e-17 (1.4e-16),
@@ -33,6 +33,17 @@
 // Hops whose half spinor is zero contribute nothing.  Infinities, NaN,
 // half spinors below 2^-523 or from 2^477 in magnitude, and links outside
 // 2^-60 .. 2^60 send the site to the plain FP64 hopping term (fx_site_f64).
+//
+// Components.  One last place serves all numbers that share an exponent, so a
+// component far below the others would keep fewer bits than in FP64 arithmetic,
+// whose errors are relative to the component's own terms.  Every real sum
+// therefore carries the sum T of the absolute values of its hops' transported
+// numbers (at most that of its products' absolute values), and a site with a sum of
+// T < 2^54.5 last places goes to the plain FP64 hop too.  From there on the errors,
+// at most 35 last places (2.8 per hop and one per alignment; 1.1 in the root mean
+// square), are below 13 2^-53 T (0.4 2^-53 T), as those of FP64 arithmetic are.  A
+// Gaussian field on any links has the eight terms of a component that small at one
+// site in 10^7; a component without a nonzero term is zero either way.
 #pragma once
 
 #include "dslash.cuh"
@@ -55,6 +66,8 @@ constexpr int FX_MIN_EXP = 500, FX_MAX_EXP = 1500;
 constexpr int FX_BAD_EXP = -32768;     // link exponent of a link that cannot be converted
 constexpr int FX_LINK_EXP = 60;
 constexpr int FX_PLANES = 9;
+// the least sum of a component's absolute values, in units of 2^48 last places
+constexpr int FX_MIN_MAG = 90;
 
 // c + a b, 32 x 32 -> 64 bits signed, as the carry pair that assembles into
 // one IMAD.WIDE (mad.wide.s32 becomes a product and a separate addition, and
@@ -94,12 +107,12 @@ __device__ __forceinline__ void fx_split(long long f, int &l1, int &l0) {
     l1 = (int)(f >> 32) + (int)((unsigned)l0 >> 31);
 }
 
-// v 2^(x - 1079) rounded to FP64 (x in about 500 .. 1600): the conversion
+// v 2^(x - 1080) rounded to FP64 (x in about 500 .. 1600): the conversion
 // instruction, then the exponent field
 __device__ __forceinline__ double fx_to_double(long long v, int x) {
     const double d = __ll2double_rn(v);
     const int hi = __double2hiint(d);
-    return __hiloint2double(v == 0 ? 0 : hi + (x - 1079) * (1 << 20), __double2loint(d));
+    return __hiloint2double(v == 0 ? 0 : hi + (x - 1080) * (1 << 20), __double2loint(d));
 }
 
 // H in at one site in FP64 arithmetic (the generic hop): the sites that the
@@ -295,6 +308,36 @@ __device__ __forceinline__ void fx_accumulate(long long a[6], long long b[6], co
     }
 }
 
+// |re|, |im| (one less for negative ones) in units of 2^48, in the halves of a
+// word: at most 2.46 2^10 of a hop, 2.46 2^13 of a component's eight
+__device__ __forceinline__ unsigned fx_mag(long long re, long long im) {
+    const unsigned hr = (unsigned)((unsigned long long)re >> 32);
+    const unsigned hi = (unsigned)((unsigned long long)im >> 32);
+    unsigned m, s;
+    asm("prmt.b32 %0, %1, %2, 0x7632;" : "=r"(m) : "r"(hr), "r"(hi));
+    asm("prmt.b32 %0, %1, %2, 0xFFBB;" : "=r"(s) : "r"(hr), "r"(hi));   // the signs
+    return m ^ s;
+}
+// both halves shifted right by d >= 0
+__device__ __forceinline__ unsigned fx_mag_shift(unsigned t, int d) {
+    return d > 15 ? 0u : (t >> d) & ((0xFFFFu >> d) * 0x10001u);
+}
+// whether both halves reach FX_MIN_MAG
+__device__ __forceinline__ bool fx_mag_ok(unsigned t) {
+    return ((t + (0x8000u - FX_MIN_MAG) * 0x10001u) & 0x80008000u) == 0x80008000u;
+}
+// ta, tb (a word per colour, 32 apart) += the magnitudes of the terms that
+// fx_accumulate adds to a and b
+__device__ __forceinline__ void fx_magnitudes(unsigned *ta, unsigned *tb, const long long u[6],
+                                              int mu) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const unsigned m = fx_mag(u[2 * i], u[2 * i + 1]);
+        atomicAdd(ta + 32 * i, m);
+        atomicAdd(tb + 32 * i, (mu & 1) ? m : __byte_perm(m, 0, 0x1032));
+    }
+}
+
 __device__ __forceinline__ bool fx_out_of_range(int eb, int eu) {
     return eb < FX_MIN_EXP || eb > FX_MAX_EXP || eu == FX_BAD_EXP;
 }
@@ -335,6 +378,10 @@ constexpr int FX_SITES = 32;      // sites per block
 
 struct FxShared {
     long long v[2][4][6][32];
+    // Magnitudes: words of one thread at a time, in shared memory because six
+    // registers more spill (197 against 210 us at 24^3 x 48); its additions need no
+    // result, so they go out as atomics (200 as loads and stores).
+    unsigned ta[4][3][32], tb[4][3][32];
     int xa[2][4][32];
 };
 
@@ -348,10 +395,13 @@ __device__ __forceinline__ void fx_site(const FxArgs &A, unsigned h, int w, FxSh
     site_coords(A.d.g, h, A.d.parity, c);
     const bool any_exp = __ldg(A.any_exp) != 0;
     long long a[6], b[6];
+    unsigned *ta = &sh.ta[w][0][lane], *tb = &sh.tb[w][0][lane];   // as a and b
 #pragma unroll
     for (int i = 0; i < 6; ++i) a[i] = b[i] = 0;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) ta[32 * i] = tb[32 * i] = 0;
     int xa = -(1 << 20);
-    bool bad = false;
+    bool bad = false, any_a = false, any_b = false;   // any term in a, in b
 #pragma unroll 1
     for (int mu = 0; mu < 4; ++mu) {
         if (mu == 2) {   // row k goes on with spin 2 + k
@@ -363,15 +413,21 @@ __device__ __forceinline__ void fx_site(const FxArgs &A, unsigned h, int w, FxSh
             const int xo = sh.xa[0][w ^ 1][lane];
 #pragma unroll
             for (int i = 0; i < 6; ++i) b[i] = sh.v[0][w ^ 1][i][lane];
+            tb = &sh.tb[w ^ 1][0][lane];
+            any_b = xo >= 0;
             if (xo != xa) {   // b comes in the other row's units
                 const int x = max(xo, xa);
                 if (xa >= 0) {
 #pragma unroll
                     for (int i = 0; i < 6; ++i) a[i] = sar64(a[i], x - xa);
+#pragma unroll
+                    for (int i = 0; i < 3; ++i) ta[32 * i] = fx_mag_shift(ta[32 * i], x - xa);
                 }
                 if (xo >= 0) {
 #pragma unroll
                     for (int i = 0; i < 6; ++i) b[i] = sar64(b[i], x - xo);
+#pragma unroll
+                    for (int i = 0; i < 3; ++i) tb[32 * i] = fx_mag_shift(tb[32 * i], x - xo);
                 }
                 xa = x;
             }
@@ -398,22 +454,41 @@ __device__ __forceinline__ void fx_site(const FxArgs &A, unsigned h, int w, FxSh
                     a[i] = sar64(a[i], d);
                     b[i] = sar64(b[i], d);
                 }
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    ta[32 * i] = fx_mag_shift(ta[32 * i], d);
+                    tb[32 * i] = fx_mag_shift(tb[32 * i], d);
+                }
             }
             xa = x;
         }
+        any_a = any_b = true;
         long long u[6];
         fx_product(U, r, ((unsigned)(xa - eu) << 20) | 0xFFFFFu, fwd, u);
         fx_accumulate(a, b, u, mu, fx_row_neg(mu, k));
+        fx_magnitudes(ta, tb, u, mu);
     }
-    // the forward warp keeps a and gives b, the backward warp the reverse; a
-    // bad site is marked in the exponent
+    // the forward warp keeps a and gives b, the backward warp the reverse; what
+    // has no term comes without an exponent, a bad site is marked in it
+    const int xg = (fwd ? any_b : any_a) ? xa : -1;
+    const int xk = (fwd ? any_a : any_b) ? xa : -1;
 #pragma unroll
     for (int i = 0; i < 6; ++i) sh.v[1][w][i][lane] = fwd ? b[i] : a[i];
-    sh.xa[1][w][lane] = bad ? (1 << 24) : xa;
+    sh.xa[1][w][lane] = bad ? (1 << 24) : xg;
     __syncwarp();
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < 4; ++q) bad = bad || sh.xa[1][q][lane] == (1 << 24);
+    const int xb = sh.xa[1][w ^ 2][lane], xm = max(xk, xb);
+    if (!bad && xm >= 0) {
+        // the warp's own and the partner's, the one with the smaller exponent shifted
+        const unsigned *to = fwd ? &sh.ta[w][0][lane] : &sh.tb[w ^ 1][0][lane];
+        const unsigned *tg = fwd ? &sh.ta[w ^ 2][0][lane] : &sh.tb[w ^ 3][0][lane];
+        const unsigned *big = xk >= xb ? to : tg, *small = xk >= xb ? tg : to;
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+            bad = bad || !fx_mag_ok(big[32 * i] + fx_mag_shift(small[32 * i], xm - min(xk, xb)));
+    }
     if (bad) {
         double t[24];
         fx_fallback(A, h, t);
@@ -425,15 +500,14 @@ __device__ __forceinline__ void fx_site(const FxArgs &A, unsigned h, int w, FxSh
         }
         return;
     }
-    const int xb = sh.xa[1][w ^ 2][lane], xm = max(xa, xb);
     // opposite projectors: spins 2, 3 take forward minus backward, times the
     // forward one's sign (-1 for H, +1 for H^dag)
 #pragma unroll
     for (int i = 0; i < 6; ++i) {
         long long got = sh.v[1][w ^ 2][i][lane], own = fwd ? a[i] : b[i];
-        if (xa != xb) {
+        if (xk != xb) {
             got = xb >= 0 ? sar64(got, xm - xb) : 0;
-            own = xa >= 0 ? sar64(own, xm - xa) : 0;
+            own = xk >= 0 ? sar64(own, xm - xk) : 0;
         }
         const long long sum = fwd ? own + got : A.dagger ? got - own : own - got;
         v[i] = fx_to_double(sum, xm);
@@ -492,43 +566,42 @@ __device__ __forceinline__ void fx_site_wide(const FxArgs &A, unsigned h, int w,
     __syncthreads();
     if (w >= 12) return;
     const int s = w & 3, cc = w >> 2;
-    int xm = -1;
-#pragma unroll
-    for (int t = 0; t < 16; ++t) xm = max(xm, sh.xa[t][lane]);
-    if (xm == 1 << 24) {
-        double t[24];
-        fx_fallback(A, h, t);
-#pragma unroll
-        for (int j = 0; j < 12; ++j)
-            if (j == w) { v[0] = t[2 * j]; v[1] = t[2 * j + 1]; }
-        return;
-    }
-    xm = -1;
-    int xt[8];
+    int xm = -1, xt[8];
 #pragma unroll
     for (int t = 0; t < 8; ++t) {   // t = 2 mu + backward
         const int k = s < 2 ? s : t < 4 ? 3 - s : s - 2;
         xt[t] = sh.xa[2 * t + k][lane];
         xm = max(xm, xt[t]);
     }
-    long long re = 0, im = 0;
+    long long re = 0, im = 0, mr = 0, mi = 0;   // and the sums of the magnitudes
+    bool bad = xm == 1 << 24;
+    if (!bad) {
 #pragma unroll
-    for (int t = 0; t < 8; ++t) {
-        if (xt[t] < 0) continue;
-        const int mu = t >> 1, k = s < 2 ? s : t < 4 ? 3 - s : s - 2;
-        const long long ur = sar64(sh.u[2 * t + k][2 * cc][lane], xm - xt[t]);
-        const long long ui = sar64(sh.u[2 * t + k][2 * cc + 1][lane], xm - xt[t]);
-        if (s < 2) {
-            re += ur;
-            im += ui;
-        } else {
-            // -i u (x, z) or u (y, t), with the row's sign; H: backward minus
-            // forward, H^dag the reverse
-            const bool minus = fx_row_neg(mu, k) != ((t & 1) == (A.dagger != 0 ? 1 : 0));
-            const long long br = (mu & 1) ? ur : ui, bi = (mu & 1) ? ui : -ur;
+        for (int t = 0; t < 8; ++t) {
+            if (xt[t] < 0) continue;
+            const int mu = t >> 1, k = s < 2 ? s : t < 4 ? 3 - s : s - 2;
+            const long long ur = sar64(sh.u[2 * t + k][2 * cc][lane], xm - xt[t]);
+            const long long ui = sar64(sh.u[2 * t + k][2 * cc + 1][lane], xm - xt[t]);
+            // -i u (x, z) or u (y, t) for spins 2 and 3, with the row's sign; H:
+            // backward minus forward, H^dag the reverse
+            const bool swap = s >= 2 && (mu & 1) == 0;
+            const bool minus =
+                s >= 2 && fx_row_neg(mu, k) != ((t & 1) == (A.dagger != 0 ? 1 : 0));
+            const long long br = swap ? ui : ur, bi = swap ? -ur : ui;
             re += minus ? -br : br;
             im += minus ? -bi : bi;
+            mr += br ^ (br >> 63);
+            mi += bi ^ (bi >> 63);
         }
+        bad = xm >= 0 && ((mr >> 48) < FX_MIN_MAG || (mi >> 48) < FX_MIN_MAG);
+    }
+    if (bad) {
+        double t[24];
+        fx_fallback(A, h, t);
+#pragma unroll
+        for (int j = 0; j < 12; ++j)
+            if (j == w) { v[0] = t[2 * j]; v[1] = t[2 * j + 1]; }
+        return;
     }
     v[0] = fx_to_double(re, xm);
     v[1] = fx_to_double(im, xm);
