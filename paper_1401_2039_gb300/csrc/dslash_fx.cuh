@@ -6,9 +6,8 @@
 // bound by that pipe: 1673 us at 32^3 x 64, 558 us at 24^3 x 48, 131 us at
 // 16^3 x 32, 55 us at 4^4.  Here the SU(3) products and the sum over the eight
 // hops run on the integer pipes; FP64 keeps the spin projection (12 additions
-// per hop) and the epilogue: 516, 172, 41 and 8 us.  What bounds it now: issue
-// (46 % active at the 20 warps per SM that 96 registers allow), with the FP64
-// pipe 53 % busy and DRAM at 40 %.
+// per hop) and the epilogue: 582, 193, 46 and 8 us (516, 172, 41 and 8 without the
+// check of the components, see below).
 //
 // Numbers.  A link element is u = Fu 2^(eu - 62) with a 62-bit integer Fu and
 // one exponent eu per link: |u| <= 2^eu, and the absolute values of the six
@@ -32,14 +31,14 @@
 //
 // Hops whose half spinor is zero contribute nothing.  Infinities, NaN,
 // half spinors below 2^-523 or from 2^477 in magnitude, and links outside
-// 2^-60 .. 2^60 send the site to the plain FP64 hopping term (fx_site_f64).
+// 2^-60 .. 2^60 leave the site to FP64 arithmetic (fx_site_f64, fx_number_f64).
 //
 // Components.  One last place serves all numbers that share an exponent, so a
 // component far below the others would keep fewer bits than in FP64 arithmetic,
 // whose errors are relative to the component's own terms.  Every real sum
 // therefore carries the sum T of the absolute values of its hops' transported
 // numbers (at most that of its products' absolute values), and a site with a sum of
-// T < 2^54.5 last places goes to the plain FP64 hop too.  From there on the errors,
+// T < 2^54.5 last places is left to FP64 arithmetic too.  From there on the errors,
 // at most 35 last places (2.8 per hop and one per alignment; 1.1 in the root mean
 // square), are below 13 2^-53 T (0.4 2^-53 T), as those of FP64 arithmetic are.  A
 // Gaussian field on any links has the eight terms of a component that small at one
@@ -113,19 +112,6 @@ __device__ __forceinline__ double fx_to_double(long long v, int x) {
     const double d = __ll2double_rn(v);
     const int hi = __double2hiint(d);
     return __hiloint2double(v == 0 ? 0 : hi + (x - 1080) * (1 << 20), __double2loint(d));
-}
-
-// H in at one site in FP64 arithmetic (the generic hop): the sites that the
-// fixed-point form does not cover
-template <int RECON, int DAG>
-__device__ __noinline__ void fx_site_f64(const DslashArgs<double> &a, long h, double *acc) {
-    int c[4];
-    site_coords(a.g, h, a.parity, c);
-    for (int k = 0; k < 24; ++k) acc[k] = 0;
-    hop_pair<double, double, RECON, 0, DAG>(a, c, h, acc);
-    hop_pair<double, double, RECON, 1, DAG>(a, c, h, acc);
-    hop_pair<double, double, RECON, 2, DAG>(a, c, h, acc);
-    hop_pair<double, double, RECON, 3, DAG>(a, c, h, acc);
 }
 
 __device__ __forceinline__ double2 ld_nc_d2(const char *p) {
@@ -352,23 +338,55 @@ __device__ __forceinline__ bool fx_wraps(const FxArgs &A, int mu, bool wrap) {
     return (A.d.phase_on >> mu & 1u) && __any_sync(__activemask(), wrap) && wrap;
 }
 
-// the site by the plain FP64 hop
-__device__ __forceinline__ void fx_fallback(const FxArgs &A, unsigned h, double t[24]) {
-    if (A.recon == 12) {
-        if (A.dagger) fx_site_f64<12, 1>(A.d, h, t);
-        else fx_site_f64<12, 0>(A.d, h, t);
+// FP64 arithmetic, for the sites that the fixed-point form leaves to it.  Element
+// (i, j) of the matrix of the hop's product, U forward, its adjoint backward
+// (12-real links: row 2 is rebuilt as in load_link)
+template <int RECON>
+__device__ __forceinline__ double2 fx_elem_f64(const FxArgs &A, unsigned site, int mu, bool fwd,
+                                               int i, int j) {
+    const size_t plane = (size_t)A.d.g.stride * 16;
+    const char *base = (fwd ? A.d.gauge_out : A.d.gauge_in) + mu * A.d.dir_bytes + site * 16u;
+    const int r = fwd ? i : j, c = fwd ? j : i;
+    double2 e;
+    if (RECON == 18 || r < 2) {
+        e = ld_nc_d2(base + (3 * r + c) * plane);
     } else {
-        if (A.dagger) fx_site_f64<18, 1>(A.d, h, t);
-        else fx_site_f64<18, 0>(A.d, h, t);
+        const int c1 = c == 2 ? 0 : c + 1, c2 = c == 0 ? 2 : c - 1;
+        const double2 a1 = ld_nc_d2(base + c1 * plane), a2 = ld_nc_d2(base + c2 * plane);
+        const double2 b1 = ld_nc_d2(base + (3 + c1) * plane), b2 = ld_nc_d2(base + (3 + c2) * plane);
+        e.x = a1.x * b2.x; e.x -= a1.y * b2.y; e.x -= a2.x * b1.x; e.x += a2.y * b1.y;
+        e.y = a2.x * b1.y; e.y += a2.y * b1.x; e.y -= a1.x * b2.y; e.y -= a1.y * b2.x;
     }
+    // (on the sign bit: a conditional negation of a double is an FP64 instruction)
+    return make_double2(e.x, __hiloint2double(__double2hiint(e.y) ^ (fwd ? 0 : (int)0x80000000u),
+                                              __double2loint(e.y)));
+}
+// colour i of the transported row r
+template <int RECON>
+__device__ __forceinline__ double2 fx_colour_f64(const FxArgs &A, unsigned site, int mu, bool fwd,
+                                                 int i, const double r[6]) {
+    double2 u;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const double2 e = fx_elem_f64<RECON>(A, site, mu, fwd, i, j);
+        u.x = j == 0 ? pmul(e.x, r[0]) : pmac(e.x, r[2 * j], u.x);
+        u.y = j == 0 ? pmul(e.x, r[1]) : pmac(e.x, r[2 * j + 1], u.y);
+        u.x = pmsub(e.y, r[2 * j + 1], u.x);
+        u.y = pmac(e.y, r[2 * j], u.y);
+    }
+    return u;
+}
+__device__ __forceinline__ double2 fx_phase_f64(const FxArgs &A, int mu, bool fwd, double2 u) {
+    const double pr = A.d.ph[2 * mu], pi = fwd ? A.d.ph[2 * mu + 1] : -A.d.ph[2 * mu + 1];
+    return make_double2(u.x * pr - u.y * pi, u.x * pi + u.y * pr);
 }
 
 // Work split: the four warps of a 128-thread block take 32 consecutive sites,
 // warp (k, dir) row k of the half spinors of their four forward or four
 // backward hops.  One thread per site needs 24 64-bit accumulators (152
-// registers, 12 warps per SM); it measured the same at 32^3 x 64 (518 against
-// 515 us) and loses below: 188 / 172 us at 24^3 x 48, 48 / 41 at 16^3 x 32, 24 /
-// 11 at 8^4.  Row k goes into
+// registers, 12 warps per SM); without the check of the components it measured the
+// same at 32^3 x 64 (518 against 515 us) and loses below: 188 / 172 us at 24^3 x 48,
+// 48 / 41 at 16^3 x 32, 24 / 11 at 8^4.  Row k goes into
 // spin k (accumulator a) and spin 3 - k for directions x and y, 2 + k for z
 // and t (accumulator b, exchanged between the two rows' warps in between); the
 // forward and the backward warp add up at the end, where one keeps spin k and
@@ -384,6 +402,66 @@ struct FxShared {
     unsigned ta[4][3][32], tb[4][3][32];
     int xa[2][4][32];
 };
+
+// The sites marked by any of the four warps, in FP64 arithmetic and the same split,
+// so that a site costs what it costs in the plain hop.  A hop with every site
+// marked before the first product (a field near 1e-290): 160 us at 16^3 x 32, 731
+// at 24^3 x 48; marked after the products, 165 and 740; FP64 arithmetic alone with
+// a thread per site, 131 and 563.
+// (Every thread its whole site: 442 and 2127 us.)  Every thread of the block calls it.
+template <int RECON>
+__device__ __noinline__ void fx_site_f64(const FxArgs &A, unsigned h, int w, FxShared &sh, bool bad,
+                                         double v[6]) {
+    const int lane = threadIdx.x & 31, k = w & 1;
+    const bool fwd = w < 2;
+    sh.xa[0][w][lane] = bad;
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) bad = bad || sh.xa[0][q][lane] != 0;
+    int c[4];
+    site_coords(A.d.g, h, A.d.parity, c);
+    double a[6], b[6];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) a[i] = b[i] = 0;
+#pragma unroll 1
+    for (int mu = 0; mu < 4; ++mu) {
+        if (mu == 2) {   // row k goes on with spin 2 + k
+#pragma unroll
+            for (int i = 0; i < 6; ++i) sh.v[0][w][i][lane] = __double_as_longlong(b[i]);
+            __syncwarp();
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < 6; ++i) b[i] = __longlong_as_double(sh.v[0][w ^ 1][i][lane]);
+        }
+        bool wrap;
+        const unsigned hn = fx_neighbour(A.d.g, h, c, mu, fwd, wrap), site = fwd ? h : hn;
+        wrap = wrap && bad && (A.d.phase_on >> mu & 1u);
+        const bool phase = __any_sync(0xffffffffu, wrap);   // (a branch, as in fx_wraps)
+        if (!bad) continue;
+        double r[6];
+        fx_half_row(A, hn, mu, k, fwd, r);
+        const double sb = fx_row_neg(mu, k) ? -1.0 : 1.0;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            double2 u = fx_colour_f64<RECON>(A, site, mu, fwd, i, r);
+            if (phase && wrap) u = fx_phase_f64(A, mu, fwd, u);
+            a[2 * i] += u.x;
+            a[2 * i + 1] += u.y;
+            b[2 * i] = fma(sb, (mu & 1) ? u.x : u.y, b[2 * i]);
+            b[2 * i + 1] = fma((mu & 1) ? sb : -sb, (mu & 1) ? u.y : u.x, b[2 * i + 1]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 6; ++i) sh.v[1][w][i][lane] = __double_as_longlong(fwd ? b[i] : a[i]);
+    __syncwarp();
+    __syncthreads();
+    if (!bad) return;
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+        const double got = __longlong_as_double(sh.v[1][w ^ 2][i][lane]), own = fwd ? a[i] : b[i];
+        v[i] = fwd ? own + got : A.dagger ? got - own : own - got;
+    }
+}
 
 // every thread of the block calls it, the four warps of one lane on the same
 // site h: v = spin k (forward warps) or 2 + k of H in, [colour][re, im]
@@ -489,17 +567,6 @@ __device__ __forceinline__ void fx_site(const FxArgs &A, unsigned h, int w, FxSh
         for (int i = 0; i < 3; ++i)
             bad = bad || !fx_mag_ok(big[32 * i] + fx_mag_shift(small[32 * i], xm - min(xk, xb)));
     }
-    if (bad) {
-        double t[24];
-        fx_fallback(A, h, t);
-        const int sp = fwd ? k : 2 + k;
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            v[2 * i] = t[8 * i + 2 * sp];
-            v[2 * i + 1] = t[8 * i + 2 * sp + 1];
-        }
-        return;
-    }
     // opposite projectors: spins 2, 3 take forward minus backward, times the
     // forward one's sign (-1 for H, +1 for H^dag)
 #pragma unroll
@@ -512,6 +579,15 @@ __device__ __forceinline__ void fx_site(const FxArgs &A, unsigned h, int w, FxSh
         const long long sum = fwd ? own + got : A.dagger ? got - own : own - got;
         v[i] = fx_to_double(sum, xm);
     }
+    __syncwarp();
+    if (!__syncthreads_or(bad)) return;
+    double t[6];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) t[i] = v[i];
+    if (A.recon == 12) fx_site_f64<12>(A, h, w, sh, bad, t);
+    else fx_site_f64<18>(A, h, w, sh, bad, t);
+#pragma unroll
+    for (int i = 0; i < 6; ++i) v[i] = t[i];
 }
 
 // The same with one hop per warp, for lattices whose blocks leave the chip nearly
@@ -533,6 +609,31 @@ struct FxWideShared {
     long long u[16][6][32];
     int xa[16][32];      // exponent, negative: no term, 1 << 24: a bad site
 };
+
+// complex number 4 cc + s of H in at site h in FP64 arithmetic
+template <int RECON>
+__device__ __noinline__ double2 fx_number_f64(const FxArgs &A, unsigned h, int cc, int s) {
+    int c[4];
+    site_coords(A.d.g, h, A.d.parity, c);
+    double2 v = make_double2(0.0, 0.0);
+#pragma unroll 1
+    for (int t = 0; t < 8; ++t) {
+        const int mu = t >> 1, k = s < 2 ? s : t < 4 ? 3 - s : s - 2;
+        const bool fwd = (t & 1) == 0;
+        bool wrap;
+        const unsigned hn = fx_neighbour(A.d.g, h, c, mu, fwd, wrap), site = fwd ? h : hn;
+        double r[6];
+        fx_half_row(A, hn, mu, k, fwd, r);
+        double2 u = fx_colour_f64<RECON>(A, site, mu, fwd, cc, r);
+        if (wrap && (A.d.phase_on >> mu & 1u)) u = fx_phase_f64(A, mu, fwd, u);
+        const bool swap = s >= 2 && (mu & 1) == 0;
+        const bool minus = s >= 2 && fx_row_neg(mu, k) != (fwd == (A.dagger == 0));
+        const double sg = minus ? -1.0 : 1.0;
+        v.x = fma(sg, swap ? u.y : u.x, v.x);
+        v.y = fma(swap ? -sg : sg, swap ? u.x : u.y, v.y);
+    }
+    return v;
+}
 
 // v = complex number w (w < 12) of H in at site h, [re, im]
 __device__ __forceinline__ void fx_site_wide(const FxArgs &A, unsigned h, int w, FxWideShared &sh,
@@ -596,11 +697,10 @@ __device__ __forceinline__ void fx_site_wide(const FxArgs &A, unsigned h, int w,
         bad = xm >= 0 && ((mr >> 48) < FX_MIN_MAG || (mi >> 48) < FX_MIN_MAG);
     }
     if (bad) {
-        double t[24];
-        fx_fallback(A, h, t);
-#pragma unroll
-        for (int j = 0; j < 12; ++j)
-            if (j == w) { v[0] = t[2 * j]; v[1] = t[2 * j + 1]; }
+        const double2 f = A.recon == 12 ? fx_number_f64<12>(A, h, cc, s)
+                                        : fx_number_f64<18>(A, h, cc, s);
+        v[0] = f.x;
+        v[1] = f.y;
         return;
     }
     v[0] = fx_to_double(re, xm);
