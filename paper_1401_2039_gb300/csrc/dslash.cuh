@@ -1190,8 +1190,10 @@ constexpr DslashCfg DSLASH_CFGS[N_DSLASH_CFG] = {
     {128, 1, 2, 0}, {128, 5, 1, 2}, {128, 6, 1, 1}, {128, 6, 1, 2},
     {SPLIT_BLOCK, 3, 1, 0, 1}};
 // whether candidate k is distinct for storage precision prec (staging
-// applies to 16-bit storage only; elsewhere it repeats an unstaged entry)
+// applies to 16-bit storage only; elsewhere it repeats an unstaged entry; the
+// kernel of one warp per hop takes 4-byte and 16-bit storage)
 inline bool dslash_cfg_applies(int k, int prec) {
+    if (DSLASH_CFGS[k].split) return prec == WD_F32 || prec == WD_F16 || prec == WD_BF16;
     return !DSLASH_CFGS[k].stage || prec == WD_F16 || prec == WD_BF16;
 }
 // The double-float hopping term (one site per thread, a loop over the hops)
@@ -1228,8 +1230,11 @@ void launch_any_cfg(int cfg, const DslashArgs<R> &a, cudaStream_t s) {
     case 6: launch_cfg<S, R, RECON, DAG, EPI, NORM, 6>(a, s); break;
     case 7: launch_cfg<S, R, RECON, DAG, EPI, NORM, 7>(a, s); break;
     case 8:
-        if constexpr (sizeof(S) <= 4) launch_cfg<S, R, RECON, DAG, EPI, NORM, 8>(a, s);
-        break;
+        if constexpr (sizeof(S) <= 4) {
+            launch_cfg<S, R, RECON, DAG, EPI, NORM, 8>(a, s);
+            break;
+        }   // (8-byte storage: as candidate 0)
+        [[fallthrough]];
     default: launch_cfg<S, R, RECON, DAG, EPI, NORM, 0>(a, s); break;
     }
 }
