@@ -27,7 +27,11 @@
  * The caller owns every array it passes; calls never keep a pointer to
  * them.  The operator handle owns its packed copies (structure-of-arrays,
  * even-odd ordered, in its storage precision) and all workspace, allocated
- * by wd_op_create; apply and solve calls allocate nothing.
+ * by wd_op_create; apply and solve calls allocate nothing.  Links held in FP64
+ * (WD_F64 handles, FP64 residuals) get a fixed-point copy beside them, 18 reals
+ * per link (twice for a WD_F64 handle with recon 12), which the hopping term runs
+ * on, when it takes at most a quarter of the device memory that is free after all
+ * else; without it the hopping term runs in FP64 arithmetic.
  *
  * Streams: every call is ordered after the work already queued on the
  * stream given to wd_op_create (NULL = the legacy default stream) and the

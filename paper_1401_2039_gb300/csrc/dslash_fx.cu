@@ -173,9 +173,7 @@ cudaError_t launch_gauge_fx(const GaugeSet &gs, const Geom &g, cudaStream_t s) {
 
 cudaError_t launch_dslash_fx(const DslashLaunch &L, cudaStream_t s) {
     const GaugeSet &gs = *L.gauge;
-    // (the byte offsets within a plane are 32-bit; a handle of 2^28 sites per
-    // parity would need over 1 TB)
-    if (!gs.fx[0] || L.g.stride >= (1L << 28)) return cudaErrorInvalidValue;
+    if (!gs.fx[0]) return cudaErrorInvalidValue;
     FxArgs A;
     cudaError_t e = fill_dslash_args<double>(L, A.d);
     if (e != cudaSuccess) return e;

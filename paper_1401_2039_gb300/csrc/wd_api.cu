@@ -15,7 +15,7 @@ namespace wd {
 #define WD_DECL(P)                                                                         \
     cudaError_t launch_dslash_##P##_r18(const DslashLaunch &L, cudaStream_t s);            \
     cudaError_t launch_dslash_##P##_r12(const DslashLaunch &L, cudaStream_t s);
-WD_DECL(f32) WD_DECL(f16) WD_DECL(bf16)
+WD_DECL(f64) WD_DECL(f32) WD_DECL(f16) WD_DECL(bf16)
 #undef WD_DECL
 cudaError_t launch_dslash_df64_r18(const DslashLaunch &L, cudaStream_t s);
 cudaError_t launch_dslash_df64f32_r18(const DslashLaunch &L, cudaStream_t s);
@@ -23,7 +23,9 @@ cudaError_t launch_dslash_df64f32_r18(const DslashLaunch &L, cudaStream_t s);
 cudaError_t launch_dslash(const DslashLaunch &L, int prec, cudaStream_t s) {
     const bool r12 = L.gauge->recon == 12;
     switch (prec) {
-    case WD_F64: return launch_dslash_fx(L, s);
+    case WD_F64:
+        if (L.gauge->fx[0]) return launch_dslash_fx(L, s);
+        return r12 ? launch_dslash_f64_r12(L, s) : launch_dslash_f64_r18(L, s);
     case WD_F32: return r12 ? launch_dslash_f32_r12(L, s) : launch_dslash_f32_r18(L, s);
     case WD_F16: return r12 ? launch_dslash_f16_r12(L, s) : launch_dslash_f16_r18(L, s);
     case WD_BF16: return r12 ? launch_dslash_bf16_r12(L, s) : launch_dslash_bf16_r18(L, s);
@@ -73,14 +75,30 @@ static int dev_alloc(wd_op *op, void **p, size_t bytes) {
     return WD_OK;
 }
 
-// the fixed-point copy of an FP64 gauge set's links
+// the fixed-point copy of an FP64 gauge set's links, in one allocation, if there is
+// room for it (fx_copy_kept)
 static int alloc_fx(wd_op *op, GaugeSet &gs) {
-    gs.fx_dir_bytes = field_bytes(WD_F64, op->g.stride, 18);
-    for (int p = 0; p < 2; ++p) {
-        WD_TRY(dev_alloc(op, &gs.fx[p], 4 * gs.fx_dir_bytes));
-        WD_TRY(dev_alloc(op, (void **)&gs.fx_exp[p], sizeof(int16_t) * 4 * op->g.stride));
+    if (gs.fx[0]) return WD_OK;
+    const size_t dir = field_bytes(WD_F64, op->g.stride, 18);
+    const size_t exps = sizeof(int16_t) * 4 * op->g.stride;   // (a multiple of 512)
+    const size_t bytes = 2 * (4 * dir + exps) + sizeof(int);
+    size_t free_bytes = 0, total = 0;
+    WD_CUDA(cudaMemGetInfo(&free_bytes, &total));
+    if (!fx_copy_kept(bytes, free_bytes, op->g.stride)) return WD_OK;
+    char *p = nullptr;
+    if (cudaMalloc((void **)&p, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        return WD_OK;
     }
-    return dev_alloc(op, (void **)&gs.any_exp, sizeof(int));
+    op->allocations.push_back(p);
+    WD_CUDA(cudaMemset(p, 0, bytes));
+    gs.fx_dir_bytes = dir;
+    for (int q = 0; q < 2; ++q) {
+        gs.fx[q] = p + q * 4 * dir;
+        gs.fx_exp[q] = (int16_t *)(p + 8 * dir + q * exps);
+    }
+    gs.any_exp = (int *)(p + 8 * dir + 2 * exps);
+    return WD_OK;
 }
 
 static int fork(wd_op *op) {
@@ -178,8 +196,8 @@ static int tune_dslash(wd_op *op, int variant) {
     const int prec = hi ? op->hi_prec : op->prec;
     const int n_cfg = prec == WD_DF64 ? N_DSLASH_DF_CFG : N_DSLASH_CFG;
     auto applies = [&](int k) { return prec == WD_DF64 || dslash_cfg_applies(k, prec); };
-    if (prec == WD_F64) {   // one configuration (dslash_fx.cu)
-        op->cfg[variant] = 0;
+    if (prec == WD_F64 && (hi ? op->gauge_hi : op->gauge_lo).fx[0]) {
+        op->cfg[variant] = 0;   // one configuration (dslash_fx.cu)
         return WD_OK;
     }
     if (force) {
@@ -257,7 +275,7 @@ int wd_op_set_residual_precision(wd_op *op, int mode) {
     }
     const int want = mode ? WD_DF64 : WD_F64;
     if (want == op->hi_prec) return WD_OK;
-    if (want == WD_F64 && !op->gauge_hi.any_exp) WD_TRY(alloc_fx(op, op->gauge_hi));
+    if (want == WD_F64) WD_TRY(alloc_fx(op, op->gauge_hi));
     WD_TRY(fork(op));
     if (op->gauge_loaded) {   // both forms are 8 bytes per real: convert in place
         const long n = (long)(4 * op->gauge_hi.dir_bytes / 8);
@@ -266,7 +284,7 @@ int wd_op_set_residual_precision(wd_op *op, int mode) {
     }
     op->hi_prec = want;
     op->gauge_hi.prec = want;
-    if (op->gauge_loaded && want == WD_F64)
+    if (op->gauge_loaded && want == WD_F64 && op->gauge_hi.fx[0])
         WD_CUDA(launch_gauge_fx(op->gauge_hi, op->g, op->stream));
     if (op->gauge_loaded) WD_TRY(tune_dslash(op, 1));
     return join(op);
@@ -297,9 +315,10 @@ int wd_dslash_tuning(const wd_op *op, int hi, double *us, int n, int *block, int
     const int prec = hi == 1 ? op->hi_prec : op->prec;
     const int n_cfg = prec == WD_DF64 ? N_DSLASH_DF_CFG : N_DSLASH_CFG;
     for (int i = 0; us && i < n; ++i) us[i] = i < n_cfg ? op->tune_us[hi][i] : 0.0;
-    // the FP64 hop has one configuration, four threads per site
+    // the fixed-point hop has one configuration, four threads per site
     constexpr DslashCfg FX = {128, 5, 1, 0};
-    const DslashCfg &C = prec == WD_DF64 ? DSLASH_DF_CFGS[k] : prec == WD_F64 ? FX : DSLASH_CFGS[k];
+    const bool fx = prec == WD_F64 && (hi == 1 ? op->gauge_hi : op->gauge_lo).fx[0];
+    const DslashCfg &C = prec == WD_DF64 ? DSLASH_DF_CFGS[k] : fx ? FX : DSLASH_CFGS[k];
     if (block) *block = C.block;
     if (min_blocks) *min_blocks = C.minb;
     if (sites_per_thread) *sites_per_thread = C.spt;
@@ -378,7 +397,6 @@ static int create_impl(wd_op *op) {
     op->gauge_lo.dir_bytes = field_bytes(op->prec, g.stride, op->recon);
     for (int p = 0; p < 2; ++p)
         WD_TRY(dev_alloc(op, &op->gauge_lo.ptr[p], 4 * op->gauge_lo.dir_bytes));
-    if (op->prec == WD_F64) WD_TRY(alloc_fx(op, op->gauge_lo));
     op->hi_shared = (op->prec == WD_F64 && op->recon == 18);
     if (op->hi_shared) {
         op->gauge_hi = op->gauge_lo;
@@ -388,7 +406,6 @@ static int create_impl(wd_op *op) {
         op->gauge_hi.dir_bytes = field_bytes(op->hi_prec, g.stride, 18);
         for (int p = 0; p < 2; ++p)
             WD_TRY(dev_alloc(op, &op->gauge_hi.ptr[p], 4 * op->gauge_hi.dir_bytes));
-        if (op->hi_prec == WD_F64) WD_TRY(alloc_fx(op, op->gauge_hi));
     }
     // fields
     const size_t lo = op->lo_field_bytes(), hi = op->hi_field_bytes();
@@ -413,6 +430,10 @@ static int create_impl(wd_op *op) {
     WD_CUDA(cudaHostAlloc((void **)&op->host_consts, sizeof(double) * 4, cudaHostAllocMapped));
     WD_CUDA(cudaHostGetDevicePointer((void **)&op->sc_host_dev, op->sc_host, 0));
     WD_CUDA(cudaHostGetDevicePointer((void **)&op->host_consts_dev, op->host_consts, 0));
+    // last: the fixed-point copies take only what is left
+    if (op->prec == WD_F64) WD_TRY(alloc_fx(op, op->gauge_lo));
+    if (op->hi_shared) op->gauge_hi = op->gauge_lo;
+    else if (op->hi_prec == WD_F64) WD_TRY(alloc_fx(op, op->gauge_hi));
     WD_CUDA(cudaDeviceSynchronize());
     return WD_OK;
 }
@@ -461,10 +482,11 @@ int wd_op_set_gauge(wd_op *op, const double *U) {
     if (!op || !U) return fail(WD_ERR_ARG, "null argument to wd_op_set_gauge");
     WD_TRY(fork(op));
     WD_CUDA(launch_pack_gauge(op->gauge_lo, op->g, U, op->stream));
-    if (op->prec == WD_F64) WD_CUDA(launch_gauge_fx(op->gauge_lo, op->g, op->stream));
+    if (op->gauge_lo.fx[0]) WD_CUDA(launch_gauge_fx(op->gauge_lo, op->g, op->stream));
     if (!op->hi_shared) {
         WD_CUDA(launch_pack_gauge(op->gauge_hi, op->g, U, op->stream));
-        if (op->hi_prec == WD_F64) WD_CUDA(launch_gauge_fx(op->gauge_hi, op->g, op->stream));
+        if (op->hi_prec == WD_F64 && op->gauge_hi.fx[0])
+            WD_CUDA(launch_gauge_fx(op->gauge_hi, op->g, op->stream));
     }
     WD_TRY(tune_dslash(op, 0));
     WD_TRY(tune_dslash(op, 2));

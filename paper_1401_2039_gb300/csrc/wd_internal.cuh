@@ -588,12 +588,22 @@ struct GaugeSet {       // links of both parities, one precision/reconstruction
     int recon = 18;
     // FP64 links as fixed-point limbs for the integer hop (dslash_fx.cuh):
     // [parity] -> 4 direction blocks of 9 planes, the link exponents
-    // [direction][stride], and whether any exponent is not 0.  Null: none kept.
+    // [direction][stride], and whether any exponent is not 0.  Null: none kept,
+    // the hop runs in FP64 arithmetic (dslash.cuh).
     void *fx[2] = {nullptr, nullptr};
     size_t fx_dir_bytes = 0;
     int16_t *fx_exp[2] = {nullptr, nullptr};
     int *any_exp = nullptr;
 };
+
+// Whether the links of an FP64 gauge set get a fixed-point copy: 18 reals per link
+// beside the 18 or 12 that the set holds anyway, for a hop 2.9 times as fast.  A
+// lattice that fits without it has to go on fitting, so the copy is the last thing
+// allocated and takes at most a quarter of what is then free.  (And the kernel's
+// byte offsets within a plane are 32-bit.)
+inline bool fx_copy_kept(size_t bytes, size_t free_bytes, long stride) {
+    return stride < (1L << 28) && bytes <= free_bytes / 4;
+}
 
 enum Epilogue { EPI_PLAIN = 0, EPI_XPAY = 1 };
 
