@@ -87,11 +87,9 @@ __global__ void __launch_bounds__(FXW_BLOCK, 1) k_dslash_fx_wide(const __grid_co
 }
 
 template <int EPI, int NORM>
-void launch_fx(const FxArgs &A, cudaStream_t s) {
+void launch_fx(const FxArgs &A, bool wide, cudaStream_t s) {
     const long n = A.d.h1 - A.d.h0;
-    // By the lattice, not by the launch's range of sites, so that a hop in parts
-    // rounds as a whole one.
-    if ((A.d.g.vh + FX_SITES - 1) / FX_SITES <= FXW_MAX_BLOCKS) {
+    if (wide) {
         k_dslash_fx_wide<EPI, NORM><<<(unsigned)((n + FX_SITES - 1) / FX_SITES), FXW_BLOCK, 0, s>>>(A);
         return;
     }
@@ -188,13 +186,13 @@ cudaError_t launch_dslash_fx(const DslashLaunch &L, cudaStream_t s) {
     A.ex_in = gs.fx_exp[q];
     A.any_exp = gs.any_exp;
     if (L.red) {
-        launch_fx<EPI_XPAY, 1>(A, s);
+        launch_fx<EPI_XPAY, 1>(A, gs.fx_wide, s);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         return launch_finish_partials(*L.red, (L.g.vh + 31) / 32, s);
     }
-    if (L.epi == EPI_PLAIN) launch_fx<EPI_PLAIN, 0>(A, s);
-    else launch_fx<EPI_XPAY, 0>(A, s);
+    if (L.epi == EPI_PLAIN) launch_fx<EPI_PLAIN, 0>(A, gs.fx_wide, s);
+    else launch_fx<EPI_XPAY, 0>(A, gs.fx_wide, s);
     return cudaGetLastError();
 }
 

@@ -600,10 +600,9 @@ __device__ __forceinline__ void fx_site(const FxArgs &A, unsigned h, int w, FxSh
 // A hop, with the host's share, one warp per row and sense / one per hop:
 //   blocks    4 (4^4)   64 (8^4)   128 (8^3 x 16)   192   324 (12^4)   2048
 //   us     10.9 / 8.0  11.0 / 8.7    11.3 / 8.7   13.2 / 13.0  14.8 / 17.7  42 / 67
-// so the line lies where one block per SM ends; a block of 16 warps with 128
-// registers leaves no room for a second.
+// so the line lies where one block per SM ends (fx_one_hop_per_warp): blocks of 16
+// warps with 82 registers run one at a time on an SM.
 constexpr int FXW_BLOCK = 512;
-constexpr long FXW_MAX_BLOCKS = 152;
 
 struct FxWideShared {
     long long u[16][6][32];

@@ -92,6 +92,10 @@ static int alloc_fx(wd_op *op, GaugeSet &gs) {
     }
     op->allocations.push_back(p);
     WD_CUDA(cudaMemset(p, 0, bytes));
+    int dev = 0, sms = 0;
+    WD_CUDA(cudaGetDevice(&dev));
+    WD_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    gs.fx_wide = fx_one_hop_per_warp(op->g.vh, sms);
     gs.fx_dir_bytes = dir;
     for (int q = 0; q < 2; ++q) {
         gs.fx[q] = p + q * 4 * dir;

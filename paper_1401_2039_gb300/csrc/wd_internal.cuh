@@ -594,7 +594,14 @@ struct GaugeSet {       // links of both parities, one precision/reconstruction
     size_t fx_dir_bytes = 0;
     int16_t *fx_exp[2] = {nullptr, nullptr};
     int *any_exp = nullptr;
+    bool fx_wide = false;   // the hop's work split (fx_one_hop_per_warp)
 };
+
+// The split of the fixed-point hop that takes one hop per warp, 32 sites per block
+// of 16 warps, is for lattices of at most one such block per SM (one fits); by
+// the lattice, not by a launch's range of sites, so that a hop in parts rounds as a
+// whole one.
+inline bool fx_one_hop_per_warp(long vh, int sms) { return (vh + 31) / 32 <= sms; }
 
 // Whether the links of an FP64 gauge set get a fixed-point copy: 18 reals per link
 // beside the 18 or 12 that the set holds anyway, for a hop 2.9 times as fast.  A
