@@ -287,13 +287,16 @@ int wd_dslash_resident(wd_op *op, int in_slot, int out_parity, int dagger);
  * that ends each Schur operator of the CGNR iteration (tuned on its own: its
  * register demand differs).  us (optional, n entries) receives the
  * measured microseconds per launch of every candidate (0 for a candidate
- * that was not timed: link staging applies to FP16/BF16 storage only, FP64
- * hops have one configuration, and entries past the candidate count); block, min_blocks, sites_per_thread and
+ * that was not timed: link staging applies to FP16/BF16 storage only, hops on a
+ * fixed-point copy of FP64 links are not tuned, and entries past the candidate
+ * count); block, min_blocks, sites_per_thread and
  * staged (optional; staged = 1: the link records of the eight hops are copied
  * into shared memory at kernel start and the neighbour spinors are loaded two
  * hops ahead; staged = 2: the same with the spinors three hops ahead)
  * describe the chosen one; candidate 8 (FP32, FP16, BF16) runs one warp per hop,
- * 32 sites per block of 256 threads.  Returns its
+ * 32 sites per block of 256 threads.  The fixed-point hop takes 32 sites per block
+ * of 128 threads, or of 512 on lattices of at most one such block per SM, under
+ * index 0.  Returns its
  * index, or -1 for a null handle.  Setting WD_DSLASH_CFG=k in the
  * environment forces candidate k, WD_TUNE=0 keeps candidate 0. */
 int wd_dslash_tuning(const wd_op *op, int hi, double *us, int n, int *block, int *min_blocks,

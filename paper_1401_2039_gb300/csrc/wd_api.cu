@@ -319,10 +319,13 @@ int wd_dslash_tuning(const wd_op *op, int hi, double *us, int n, int *block, int
     const int prec = hi == 1 ? op->hi_prec : op->prec;
     const int n_cfg = prec == WD_DF64 ? N_DSLASH_DF_CFG : N_DSLASH_CFG;
     for (int i = 0; us && i < n; ++i) us[i] = i < n_cfg ? op->tune_us[hi][i] : 0.0;
-    // the fixed-point hop has one configuration, four threads per site
-    constexpr DslashCfg FX = {128, 5, 1, 0};
-    const bool fx = prec == WD_F64 && (hi == 1 ? op->gauge_hi : op->gauge_lo).fx[0];
-    const DslashCfg &C = prec == WD_DF64 ? DSLASH_DF_CFGS[k] : fx ? FX : DSLASH_CFGS[k];
+    // the fixed-point hop's (dslash_fx.cu): a warp per row and sense of 32 sites,
+    // or per row of one hop
+    constexpr DslashCfg FX = {128, 5, 1, 0}, FX_WIDE = {512, 1, 1, 0};
+    const GaugeSet &gs = hi == 1 ? op->gauge_hi : op->gauge_lo;
+    const bool fx = prec == WD_F64 && gs.fx[0];
+    const DslashCfg &C = prec == WD_DF64 ? DSLASH_DF_CFGS[k]
+                         : !fx ? DSLASH_CFGS[k] : gs.fx_wide ? FX_WIDE : FX;
     if (block) *block = C.block;
     if (min_blocks) *min_blocks = C.minb;
     if (sites_per_thread) *sites_per_thread = C.spt;
