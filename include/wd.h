@@ -298,7 +298,9 @@ int wd_dslash_resident(wd_op *op, int in_slot, int out_parity, int dagger);
  * of 128 threads, or of 512 on lattices of at most one such block per SM, under
  * index 0.  Returns its
  * index, or -1 for a null handle.  Setting WD_DSLASH_CFG=k in the
- * environment forces candidate k, WD_TUNE=0 keeps candidate 0. */
+ * environment forces candidate k, WD_TUNE=0 keeps candidate 0; links that become
+ * FP64 (wd_op_create, wd_op_set_residual_precision) while WD_DSLASH_CFG is set get no
+ * fixed-point copy, and their hops run as that candidate in FP64 arithmetic. */
 int wd_dslash_tuning(const wd_op *op, int hi, double *us, int n, int *block, int *min_blocks,
                      int *sites_per_thread, int *staged);
 

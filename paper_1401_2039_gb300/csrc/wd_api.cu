@@ -76,9 +76,10 @@ static int dev_alloc(wd_op *op, void **p, size_t bytes) {
 }
 
 // the fixed-point copy of an FP64 gauge set's links, in one allocation, if there is
-// room for it (fx_copy_kept)
+// room for it (fx_copy_kept); none while WD_DSLASH_CFG forces a candidate of
+// k_dslash
 static int alloc_fx(wd_op *op, GaugeSet &gs) {
-    if (gs.fx[0]) return WD_OK;
+    if (gs.fx[0] || getenv("WD_DSLASH_CFG")) return WD_OK;
     const size_t dir = field_bytes(WD_F64, op->g.stride, 18);
     const size_t exps = sizeof(int16_t) * 4 * op->g.stride;   // (a multiple of 512)
     const size_t bytes = 2 * (4 * dir + exps) + sizeof(int);
