@@ -332,10 +332,11 @@ __device__ __forceinline__ int fx_link_exp(const FxArgs &A, bool any_exp, unsign
     if (!any_exp) return 0;
     return (fwd ? A.ex_out : A.ex_in)[(size_t)mu * A.d.g.stride + site];
 }
-// the vote makes this a branch (as predicated instructions the FP64 products
-// of the phase would take the pipe in every hop)
+// The vote, to which every lane of the warp comes in every hop, makes this a branch
+// (as predicated instructions the FP64 products of the phase would take the pipe in
+// every hop).
 __device__ __forceinline__ bool fx_wraps(const FxArgs &A, int mu, bool wrap) {
-    return (A.d.phase_on >> mu & 1u) && __any_sync(__activemask(), wrap) && wrap;
+    return (A.d.phase_on >> mu & 1u) && __any_sync(0xffffffffu, wrap) && wrap;
 }
 
 // FP64 arithmetic, for the sites that the fixed-point form leaves to it.  Element
