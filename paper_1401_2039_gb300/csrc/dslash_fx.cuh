@@ -674,7 +674,8 @@ __device__ __forceinline__ void fx_site_wide(const FxArgs &A, unsigned h, int w,
         xt[t] = sh.xa[2 * t + k][lane];
         xm = max(xm, xt[t]);
     }
-    long long re = 0, im = 0, mr = 0, mi = 0;   // and the sums of the magnitudes
+    long long re = 0, im = 0;
+    int mr = 0, mi = 0;   // the sums of the absolute values, in units of 2^32
     bool bad = xm == 1 << 24;
     if (!bad) {
 #pragma unroll
@@ -691,10 +692,11 @@ __device__ __forceinline__ void fx_site_wide(const FxArgs &A, unsigned h, int w,
             const long long br = swap ? ui : ur, bi = swap ? -ur : ui;
             re += minus ? -br : br;
             im += minus ? -bi : bi;
-            mr += br ^ (br >> 63);
-            mi += bi ^ (bi >> 63);
+            const int hr = (int)(br >> 32), hi = (int)(bi >> 32);
+            mr += hr ^ (hr >> 31);
+            mi += hi ^ (hi >> 31);
         }
-        bad = xm >= 0 && ((mr >> 48) < FX_MIN_MAG || (mi >> 48) < FX_MIN_MAG);
+        bad = xm >= 0 && min(mr, mi) < FX_MIN_MAG << 16;
     }
     if (bad) {
         const double2 f = A.recon == 12 ? fx_number_f64<12>(A, h, cc, s)
