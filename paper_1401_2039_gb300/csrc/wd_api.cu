@@ -500,6 +500,9 @@ int wd_op_set_gauge(wd_op *op, const double *U) {
     WD_TRY(tune_dslash(op, 2));
     if (!op->hi_shared) WD_TRY(tune_dslash(op, 1));
     else op->cfg[1] = op->cfg[0];
+    // the links are read when the call returns: tuning waits for the stream, and
+    // hops that are not tuned must too
+    if (op->gauge_lo.fx[0]) WD_CUDA(cudaStreamSynchronize(op->stream));
     WD_TRY(join(op));
     op->gauge_loaded = true;
     return WD_OK;
