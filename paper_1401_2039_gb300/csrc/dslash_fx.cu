@@ -117,8 +117,8 @@ k_gauge_fx(Geom g, const char *links, size_t dir_bytes, char *fx, size_t fx_dir_
         const double u = fabs(U[k]);
         finite = finite && isfinite(u);
         mx = fmax(mx, u);
-        row[k / 6] += u / 2.46;
-        col[(k / 2) % 3] += u / 2.46;
+        row[k / 6] += (1 / 2.46) * u;
+        col[(k / 2) % 3] += (1 / 2.46) * u;
     }
 #pragma unroll
     for (int k = 0; k < 3; ++k) mx = fmax(mx, fmax(row[k], col[k]));
