@@ -69,7 +69,9 @@ typedef enum { WD_F64 = 0, WD_F32 = 1, WD_F16 = 2, WD_BF16 = 3 } wd_prec;
  *   kappa  hopping parameter (any real; kappa = 0 gives D = I)
  *   phase  host double[8]: (re, im) of phi_mu for mu = x, y, z, t
  *   prec   storage precision of the operator applications and of the
- *          inner solver iterations (WD_F64: plain FP64 throughout;
+ *          inner solver iterations (WD_F64: FP64 throughout, the hopping term
+ *          in block fixed-point integers at the sites where every component is
+ *          as accurate that way, relative to its own terms, as in FP64 arithmetic;
  *          WD_F32/F16/BF16: low-precision storage, FP32 arithmetic,
  *          FP64 reliable updates in wd_solve_cg)
  *   recon  18 (full links) or 12 (two rows stored, third row rebuilt as
@@ -229,7 +231,9 @@ int wd_solve_cg_host_stream(wd_op *op, int n, double *const *x_host,
  * lattices; each system keeps its own CGNR scalars, residual refreshes
  * (reliable updates, or the outer steps of defect correction: the recovery
  * mode and tolerances of the first operator apply to every system) are
- * taken together, and converged systems are frozen.  The operators must
+ * taken together, and converged systems are frozen.  Hops on FP64 fields run in
+ * FP64 arithmetic (a WD_F64 handle's own solve runs on fixed-point links, and four
+ * of them on 16^3 x 32 take half the time of a batch).  The operators must
  * outlive the batch.  Not in the paper: it batches the paper's solve (goal
  * with templates "CGNR schur") over many right-hand sides and lattices. */
 typedef struct wd_batch wd_batch;

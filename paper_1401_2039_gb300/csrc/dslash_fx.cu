@@ -27,8 +27,8 @@ __device__ __forceinline__ double2 fx_store(const DslashArgs<double> &a, long h,
 
 // The fused norm: |out|^2 per spin in FP64, the four spins and then the 32
 // sites of the block's partial in double-float.  Five blocks per SM: 96
-// registers; with four (126) or six (80, spilling) it is 6 to 11 % slower at
-// 16^3 x 32 and above and level below, so the kernel is not tuned per handle.
+// registers; with four (122) or six (80, spilling) it is 8 to 15 % slower at
+// 16^3 x 32 and above, so the kernel is not tuned per handle.
 template <int EPI, int NORM>
 __global__ void __launch_bounds__(FX_BLOCK, 5) k_dslash_fx(const __grid_constant__ FxArgs A) {
     __shared__ FxShared sh;

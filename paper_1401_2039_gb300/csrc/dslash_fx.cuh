@@ -6,8 +6,10 @@
 // bound by that pipe: 1673 us at 32^3 x 64, 558 us at 24^3 x 48, 131 us at
 // 16^3 x 32, 55 us at 4^4.  Here the SU(3) products and the sum over the eight
 // hops run on the integer pipes; FP64 keeps the spin projection (12 additions
-// per hop) and the epilogue: 582, 193, 46 and 8 us (516, 172, 41 and 8 without the
-// check of the components, see below).
+// per hop) and the epilogue: 580, 193, 46 and 8 us (516, 172, 41 and 8 without the
+// check of the components, see below).  What bounds it now: dependent issue and the
+// loads at the 20 warps per SM that 96 registers allow (issue 46 % active, FP64
+// pipe 45 % busy, DRAM 25 to 28 % on 16^3 x 32).
 //
 // Numbers.  A link element is u = Fu 2^(eu - 62) with a 62-bit integer Fu and
 // one exponent eu per link: |u| <= 2^eu, and the absolute values of the six
@@ -26,8 +28,9 @@
 // result is one rounding of a value good to about 2^-57 of the site's scale,
 // where FP64 arithmetic rounds after every operation.  Against 113-bit
 // arithmetic (relative 2-norm, 6 x 10 x 14 x 18): Gaussian fields 7.0e-17 (FP64
-// arithmetic 1.5e-16), fields falling by e^3 per time slice 7.0e-17 (1.4e-16),
-// a point source after two applications of D 5.8e-17 (7.1e-17).
+// arithmetic 1.5e-16), fields falling by e^3 per time slice 7.8e-17 (1.4e-16); a
+// point source after two applications of D (10 x 10 x 6 x 18, mean of 16) 7.2e-17
+// (8.2e-17).
 //
 // Hops whose half spinor is zero contribute nothing.  Infinities, NaN,
 // half spinors below 2^-523 or from 2^477 in magnitude, and links outside
@@ -40,9 +43,14 @@
 // numbers (at most that of its products' absolute values), and a site with a sum of
 // T < 2^54.5 last places is left to FP64 arithmetic too.  From there on the errors,
 // at most 35 last places (2.8 per hop and one per alignment; 1.1 in the root mean
-// square), are below 13 2^-53 T (0.4 2^-53 T), as those of FP64 arithmetic are.  A
-// Gaussian field on any links has the eight terms of a component that small at one
-// site in 10^7; a component without a nonzero term is zero either way.
+// square), are below 13 2^-53 T (0.4 2^-53 T), as those of FP64 arithmetic are.
+// Measured, a component's error over 2^-53 and the sum of its products' absolute
+// values, root mean square: Gaussian fields 0.13 (FP64 arithmetic 0.27), e^3 per time
+// slice 0.34 (0.43), point sources 0.36 (0.46), one colour on links within 0.1 and
+// 0.01 of 1 0.29 and 0.31 (0.33 and 0.34).  A Gaussian field has the eight terms
+// of a component that small at about one site in 10^6; fields of one colour on links
+// that hardly mix colours have them at every site (740 us at 24^3 x 48).  A row
+// without a nonzero term is zero either way.
 #pragma once
 
 #include "dslash.cuh"
@@ -598,7 +606,8 @@ __device__ __forceinline__ void fx_site(const FxArgs &A, unsigned h, int w, FxSh
 // each add the eight terms of one complex number j = 4 colour + spin, in units
 // of the largest exponent.
 //
-// A hop, with the host's share, one warp per row and sense / one per hop:
+// A hop, with the host's share, one warp per row and sense / one per hop (before
+// the check of the components):
 //   blocks    4 (4^4)   64 (8^4)   128 (8^3 x 16)   192   324 (12^4)   2048
 //   us     10.9 / 8.0  11.0 / 8.7    11.3 / 8.7   13.2 / 13.0  14.8 / 17.7  42 / 67
 // so the line lies where one block per SM ends (fx_one_hop_per_warp): blocks of 16
